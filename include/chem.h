@@ -124,11 +124,11 @@ typedef enum {
 typedef struct {
   int32_t variant;     /* chem_variant [CHEM_VARIANT_FP64] */
   int32_t max_steps;   /* attempted-step limit per cell and call [100000] */
-  int32_t block_size;  /* threads per block of the one-pass integration kernel: 32 or 64
-                          (16 warps per SM, 128 registers a thread; 32 warps at 64
-                          registers for the mixed two-register scheme), 128 (12 warps,
-                          170 registers) or 256 (8 warps, 255 registers); other values
-                          take 128 [0: 64 for the mixed variant, 128 for fp64] */
+  int32_t block_size;  /* threads per block of the one-pass integration kernel: 32, 64
+                          (16 warps per SM, 128 registers a thread; 64 registers for the
+                          mixed two-register scheme), 128 (12 warps, 170 registers; mixed
+                          two-register scheme with 9 species: 16 warps, 128 registers) or
+                          256 (8 warps, 255 registers); other values take 128 [0: 128] */
   int32_t scheme;      /* chem_scheme [CHEM_SCHEME_LSRK]; the comparators serve
                           chem_integrate and chem_integrate_host only: the batched and
                           surrogate calls of a context with another scheme return
@@ -253,7 +253,8 @@ typedef struct {
 /* Compiled shapes of the persistent kernel: (threads per CTA, minimum resident CTAs
  * per SM, hence a register cap of min(255, 65536 / (threads * CTAs))):
  * 0 = (128, 2) [default, no cap in effect], 1 = (128, 3), 2 = (128, 4), 3 = (64, 6),
- * 4 = (64, 8) [(64, 16) for the mixed variant of the 9-species library], 5 = (256, 2).
+ * 4 = (64, 8), 5 = (256, 2) for fp64; for the mixed variant 0 = (128, 4) [default], 2 = (128, 2)
+ * and 4 = (64, 16) with 9 species, 0 = (128, 3), 2 = (128, 2) with 13, the others as for fp64.
  * All run the same algorithm; the compiler contracts
  * multiply-adds per compiled kernel, so results of different shapes agree to rounding
  * (to the integration tolerance in ill-conditioned cells), not bit for bit.  Shape 0

@@ -234,6 +234,17 @@ int build_tables(const chem_mechanism *m, MechTables *t) {
   t->f.T_mid = (float)t->T_mid;
   t->f.ln_R_over_Pref = (float)t->ln_R_over_Pref;
   t->f.newton_sq = (float)t->newton_sq;
+  auto pair = [](double x, float (&o)[2]) {
+    o[0] = (float)x;
+    o[1] = (float)(x - (double)o[0]);
+  };
+  for (int r = 0; r < 2; ++r)
+    for (int k = 0; k < NSP; ++k) {
+      for (int i = 0; i < 6; ++i) pair(t->ecw[r][k][i], t->f.ecw2[r][k][i]);
+      for (int i = 0; i < 7; ++i) pair(t->gc[r][k][i], t->f.gc2[r][k][i]);
+    }
+  pair(t->T_mid, t->f.T_mid2);
+  pair(t->ln_R_over_Pref, t->f.ln_R_over_Pref2);
   return CHEM_OK;
 }
 
@@ -307,10 +318,9 @@ int chem_setup(const chem_mechanism *mech, const chem_options *opt, chem_ctx **o
     return fail(nullptr, CHEM_ERR_INVALID, "unknown variant %d", o.variant);
   if (o.max_steps < 0) return fail(nullptr, CHEM_ERR_INVALID, "max_steps < 0");
   if (o.max_steps == 0) o.max_steps = 100000;
-  // default shape of the one-pass kernel: the 64-thread blocks for the mixed variant
-  // (32 warps per SM at 64 registers, measured 3.8 % faster than 16 warps at 128), 12
-  // warps at 170 registers for fp64 (whose 128-register build spills)
-  if (o.block_size == 0) o.block_size = o.variant == CHEM_VARIANT_MIXED ? 64 : 128;
+  // default shape of the one-pass kernel: 128-thread blocks, the fastest of both variants (fp64:
+  // 12 warps per SM at 166 registers; mixed: 16 warps at 128)
+  if (o.block_size == 0) o.block_size = 128;
   if (o.scheme != CHEM_SCHEME_LSRK && o.scheme != CHEM_SCHEME_FULL_STORAGE && o.scheme != CHEM_SCHEME_RKF45)
     return fail(nullptr, CHEM_ERR_INVALID, "unknown scheme %d", o.scheme);
   for (int i = 0; i < 4; ++i)

@@ -125,13 +125,18 @@ __global__ void k_scatter(int64_t n, const uint8_t *__restrict__ bucket, int32_t
 // 65536 / (block * minb), trading registers (and spills) against resident warps.  The
 // autotuner picks among them.  Every shape runs the same algorithm, but the compiler
 // contracts multiply-adds per compiled kernel, so shapes agree to rounding, not bit for
-// bit; shape 0 (no register cap) compiles like the one-pass kernel.
+// bit; shape 0 compiles like the one-pass kernel.
 template <int V, int BLOCK, int MINB>
 __global__ void __launch_bounds__(BLOCK, MINB) k_lsrk_persistent(const __grid_constant__ MechTables mt,
                                                                  const BatchArgs a, const StepParams p,
                                                                  const int32_t *__restrict__ order,
                                                                  unsigned long long *cursor) {
-  load_math_tables();
+  if constexpr (V == CHEM_VARIANT_MIXED) {
+    load_mixed_tables<BLOCK>(mt);
+    init_mixed_cols<BLOCK>(mixed_cols<BLOCK>());
+  } else {
+    load_math_tables();
+  }
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   CellState c;
@@ -171,7 +176,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_lsrk_persistent(const __grid_co
     }
     if (__ballot_sync(FULL, cell >= 0) == 0) break;
     if (cell >= 0) {
-      if (!c.done) cell_attempt<V>(mt, c, p);
+      if (!c.done) cell_attempt<V, BLOCK>(mt, c, p);
       if (c.done) {
         if (c.status == CHEM_CELL_OK && --sub_left > 0) {
           c.t = 0.0;  // next substep from the current state; h and the T guess carry
@@ -200,23 +205,29 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_lsrk_persistent(const __grid_co
   if (a.stats) accumulate_stats(a.stats, done_cells, tot_acc, tot_rej, tot_rhs, max_steps, hist);
 }
 
-// Threads per CTA of each shape; shape 0 is the default.  Resident CTAs per SM: 2, 3, 4,
-// 6, 8 (16 for the mixed variant of the 9-species structure: 32 warps at 64 registers,
-// spilling to L1, which hides the FP64 pipe's latency by warps rather than registers),
-// 2.
+// Threads per CTA and minimum resident CTAs per SM of each shape; shape 0 is the default.  The
+// mixed variant's shapes 0 and 2 are exchanged: its default keeps 16 warps per SM (12 with
+// 13 species; its per-thread columns allow no more), which runs the ragged AMR batch in 70 ms
+// against 90 for 128 x 2 (and 83 for the 64-register shape 4).
 static constexpr int kShapeBlock[CHEM_BATCH_SHAPES] = {128, 128, 128, 64, 64, 256};
 template <int V>
-constexpr int kMinB4 = (V == CHEM_VARIANT_MIXED && NSP <= 9) ? 16 : 8;
+constexpr int kShapeMinB[CHEM_BATCH_SHAPES] = {2, 3, 4, 6, 8, 2};
+template <>
+constexpr int kShapeMinB<CHEM_VARIANT_MIXED>[CHEM_BATCH_SHAPES] = {NSP <= 9 ? 4 : 3, 3, 2, 6, NSP <= 9 ? 16 : 8, 2};
 
+template <int V, int S>
+static const void *shape_fn() {
+  return reinterpret_cast<const void *>(k_lsrk_persistent<V, kShapeBlock[S], kShapeMinB<V>[S]>);
+}
 template <int V>
 static const void *persistent_fn(int shape) {
   switch (shape) {
-    case 1: return reinterpret_cast<const void *>(k_lsrk_persistent<V, 128, 3>);
-    case 2: return reinterpret_cast<const void *>(k_lsrk_persistent<V, 128, 4>);
-    case 3: return reinterpret_cast<const void *>(k_lsrk_persistent<V, 64, 6>);
-    case 4: return reinterpret_cast<const void *>(k_lsrk_persistent<V, 64, kMinB4<V>>);
-    case 5: return reinterpret_cast<const void *>(k_lsrk_persistent<V, 256, 2>);
-    default: return reinterpret_cast<const void *>(k_lsrk_persistent<V, 128, 2>);
+    case 1: return shape_fn<V, 1>();
+    case 2: return shape_fn<V, 2>();
+    case 3: return shape_fn<V, 3>();
+    case 4: return shape_fn<V, 4>();
+    case 5: return shape_fn<V, 5>();
+    default: return shape_fn<V, 0>();
   }
 }
 static_assert(CHEM_BATCH_SHAPES == 6, "persistent_fn lists every shape");
@@ -224,6 +235,11 @@ static_assert(CHEM_BATCH_SHAPES == 6, "persistent_fn lists every shape");
 static const void *persistent_kernel(int variant, int shape) {
   return variant == CHEM_VARIANT_MIXED ? persistent_fn<CHEM_VARIANT_MIXED>(shape)
                                        : persistent_fn<CHEM_VARIANT_FP64>(shape);
+}
+
+// Dynamic shared memory of a shape: the mixed variant's per-thread columns.
+static size_t persistent_smem(int variant, int shape) {
+  return variant == CHEM_VARIANT_MIXED ? mixed_cols_bytes(kShapeBlock[shape]) : 0;
 }
 
 // Resident CTAs per SM and registers per thread of every (variant, shape), per device
@@ -243,7 +259,9 @@ cudaError_t persistent_shape(int variant, int shape, int *block, int *ctas_per_s
   if (d < 0 || g_persist_ctas[d][v][shape] == 0) {
     const void *fn = persistent_kernel(variant, shape);
     int per = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, kShapeBlock[shape], 0);
+    const size_t smem = persistent_smem(variant, shape);
+    e = allow_smem(fn, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, kShapeBlock[shape], smem);
     if (e != cudaSuccess) return e;
     cudaFuncAttributes fa{};
     e = cudaFuncGetAttributes(&fa, fn);
@@ -263,23 +281,27 @@ cudaError_t persistent_shape(int variant, int shape, int *block, int *ctas_per_s
   return cudaSuccess;
 }
 
-template <int V, int B, int M>
-static void launch_persistent_t(unsigned grid, cudaStream_t st, const MechTables &mt, const BatchArgs &a,
+template <int V, int S>
+static cudaError_t launch_shape(unsigned grid, cudaStream_t st, const MechTables &mt, const BatchArgs &a,
                                 const StepParams &p, const int32_t *order, unsigned long long *cursor) {
-  k_lsrk_persistent<V, B, M><<<grid, B, 0, st>>>(mt, a, p, order, cursor);
+  const size_t smem = persistent_smem(V, S);
+  const cudaError_t e = allow_smem(shape_fn<V, S>(), smem);
+  if (e != cudaSuccess) return e;
+  k_lsrk_persistent<V, kShapeBlock[S], kShapeMinB<V>[S]><<<grid, kShapeBlock[S], smem, st>>>(mt, a, p, order, cursor);
+  return cudaGetLastError();
 }
 
 template <int V>
-static void launch_persistent(int shape, unsigned grid, cudaStream_t st, const MechTables &mt,
-                              const BatchArgs &a, const StepParams &p, const int32_t *order,
-                              unsigned long long *cursor) {
+static cudaError_t launch_persistent(int shape, unsigned grid, cudaStream_t st, const MechTables &mt,
+                                     const BatchArgs &a, const StepParams &p, const int32_t *order,
+                                     unsigned long long *cursor) {
   switch (shape) {
-    case 1: launch_persistent_t<V, 128, 3>(grid, st, mt, a, p, order, cursor); break;
-    case 2: launch_persistent_t<V, 128, 4>(grid, st, mt, a, p, order, cursor); break;
-    case 3: launch_persistent_t<V, 64, 6>(grid, st, mt, a, p, order, cursor); break;
-    case 4: launch_persistent_t<V, 64, kMinB4<V>>(grid, st, mt, a, p, order, cursor); break;
-    case 5: launch_persistent_t<V, 256, 2>(grid, st, mt, a, p, order, cursor); break;
-    default: launch_persistent_t<V, 128, 2>(grid, st, mt, a, p, order, cursor); break;
+    case 1: return launch_shape<V, 1>(grid, st, mt, a, p, order, cursor);
+    case 2: return launch_shape<V, 2>(grid, st, mt, a, p, order, cursor);
+    case 3: return launch_shape<V, 3>(grid, st, mt, a, p, order, cursor);
+    case 4: return launch_shape<V, 4>(grid, st, mt, a, p, order, cursor);
+    case 5: return launch_shape<V, 5>(grid, st, mt, a, p, order, cursor);
+    default: return launch_shape<V, 0>(grid, st, mt, a, p, order, cursor);
   }
 }
 
@@ -289,19 +311,15 @@ cudaError_t launch_persistent_queue(int variant, const MechTables &mt, const Bat
   if (a.n <= 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
-  // the fastest shape of each variant on the ragged AMR batch: the default for fp64, the
-  // 32-warp shape 4 for mixed (127 ms against 137.5 for the default)
-  const int shape = variant == CHEM_VARIANT_MIXED ? 4 : 0;
+  const int shape = 0;  // the fastest of each variant on the ragged AMR batch
   int sms = 0, pblock = 0, per = 0, regs = 0;
   e = persistent_shape(variant, shape, &pblock, &per, &regs, &sms);
   if (e != cudaSuccess) return e;
   const int64_t cap_ctas = (int64_t)sms * per, need = (a.n + pblock - 1) / pblock;
   const unsigned grid = (unsigned)(cap_ctas < need ? cap_ctas : need);
   if (variant == CHEM_VARIANT_MIXED)
-    launch_persistent<CHEM_VARIANT_MIXED>(shape, grid, st, mt, a, p, order, cursor);
-  else
-    launch_persistent<CHEM_VARIANT_FP64>(shape, grid, st, mt, a, p, order, cursor);
-  return cudaGetLastError();
+    return launch_persistent<CHEM_VARIANT_MIXED>(shape, grid, st, mt, a, p, order, cursor);
+  return launch_persistent<CHEM_VARIANT_FP64>(shape, grid, st, mt, a, p, order, cursor);
 }
 
 cudaError_t launch_batched(int variant, const MechTables &mt, const BatchArgs &a,
@@ -331,10 +349,8 @@ cudaError_t launch_batched(int variant, const MechTables &mt, const BatchArgs &a
   const int64_t need = (a.n + pblock - 1) / pblock;
   const unsigned grid = (unsigned)(cap_ctas < need ? cap_ctas : need);
   if (variant == CHEM_VARIANT_MIXED)
-    launch_persistent<CHEM_VARIANT_MIXED>(shape, grid, st, mt, a, p, order, s.cursor);
-  else
-    launch_persistent<CHEM_VARIANT_FP64>(shape, grid, st, mt, a, p, order, s.cursor);
-  return cudaGetLastError();
+    return launch_persistent<CHEM_VARIANT_MIXED>(shape, grid, st, mt, a, p, order, s.cursor);
+  return launch_persistent<CHEM_VARIANT_FP64>(shape, grid, st, mt, a, p, order, s.cursor);
 }
 
 }  // namespace chem

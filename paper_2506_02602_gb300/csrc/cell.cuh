@@ -17,9 +17,9 @@
 // 1e-15 dt is an underflow.  A trial stage whose temperature solve fails rejects the
 // attempt with factor 1/5; a failure at stage 1 (the accepted state) ends the cell.
 //
-// Variants: V = CHEM_VARIANT_FP64, every register fp64; V = CHEM_VARIANT_MIXED, the stage
-// register U and the stage derivative F are fp32 (cell_rhs_mixed) while X, y_n, E, the
-// WRMS norm and the controller stay fp64.
+// Variants: V = CHEM_VARIANT_FP64, every register fp64; V = CHEM_VARIANT_MIXED
+// (cell_attempt_mixed), the stage register U and the stage derivative F are fp32
+// (cell_rhs_mixed) while X, y_n, E, the WRMS norm and the controller stay fp64.
 #pragma once
 
 #include <math_constants.h>
@@ -115,56 +115,67 @@ __device__ __forceinline__ void cell_begin(CellState &c, double rho, double e, d
   }
 }
 
-// One attempted step (or the end of the integration).  Sets c.done when the cell has
-// reached dt or hit a limit.
-template <int V>
-__device__ __forceinline__ void cell_attempt(const MechTables &mt, CellState &c,
-                                             const StepParams &p) {
-  constexpr bool kMixed = V == CHEM_VARIANT_MIXED;
-  using SReal = std::conditional_t<kMixed, float, double>;
+// The start of an attempt: false (with c.done, and a status where a limit was hit) when the
+// cell has reached dt or hit a limit, else h clipped to land on dt.
+__device__ __forceinline__ bool attempt_begin(CellState &c, const StepParams &p, double &h) {
   const double dt = c.dt;
-  if (!(dt - c.t > 1e-12 * dt)) { c.done = true; return; }
-  if (c.nacc + c.nrej >= p.max_steps) { c.status = CHEM_CELL_MAX_STEPS; c.done = true; return; }
-  if (c.h < 1e-15 * dt) { c.status = CHEM_CELL_H_UNDERFLOW; c.done = true; return; }
-  double h = c.h;
+  if (!(dt - c.t > 1e-12 * dt)) { c.done = true; return false; }
+  if (c.nacc + c.nrej >= p.max_steps) { c.status = CHEM_CELL_MAX_STEPS; c.done = true; return false; }
+  if (c.h < 1e-15 * dt) { c.status = CHEM_CELL_H_UNDERFLOW; c.done = true; return false; }
+  h = c.h;
   if (h > dt - c.t) h = dt - c.t;
-  double Xs[NSP], E[NSP];
-  SReal U[NSP];
+  return true;
+}
+
+// The WRMS norm's decision (Eq. 22) from the sum of the squared weighted errors: returns
+// whether the step is accepted; updates the counters, t and h.  The step factor stays IEEE
+// fp64: an explicit scheme at its stability limit grows a perturbation of h along its weakly
+// unstable modes into another rejection sequence.
+__device__ __forceinline__ bool attempt_end(CellState &c, double h, double sum) {
+  const double err = sqrt(sum * (1.0 / NSP));
+  if (!isfinite(err)) {
+    ++c.nrej;
+    c.h = h * 0.2;
+    return false;
+  }
+  const double fac = (err == 0.0) ? 5.0 : fmin(5.0, fmax(0.2, 0.9 / sqrt(sqrt(err))));
+  c.h = h * fac;
+  if (err <= 1.0) {
+    c.t += h;
+    ++c.nacc;
+    return true;
+  }
+  ++c.nrej;
+  return false;
+}
+
+// One attempted step (or the end of the integration), fp64 variant.  Sets c.done when the
+// cell has reached dt or hit a limit.
+__device__ __forceinline__ void cell_attempt_fp64(const MechTables &mt, CellState &c,
+                                                  const StepParams &p) {
+  double h;
+  if (!attempt_begin(c, p, h)) return;
+  double Xs[NSP], E[NSP], U[NSP];
 #pragma unroll
   for (int k = 0; k < NSP; ++k) {
     Xs[k] = c.X[k];
-    if constexpr (kMixed) U[k] = d2f(c.X[k]);
-    else U[k] = c.X[k];
+    U[k] = c.X[k];
     E[k] = 0.0;
   }
   int failed = 0;
   double Tacc = c.T;  // temperature of the accepted state, set by stage 1
 #pragma unroll 1
   for (int s = 0; s < 5; ++s) {
-    SReal F[NSP];
+    double F[NSP];
     ++c.nrhs;
-    bool ok;
-    if constexpr (kMixed) ok = cell_rhs_mixed(mt, U, c.rho_f, c.invRho_f, c.eR, c.T, F);
-    else ok = cell_rhs(mt, U, c.rho, c.invRho, c.eR, c.T, F);
-    if (!ok) { failed = s + 1; break; }
+    if (!cell_rhs(mt, U, c.rho, c.invRho, c.eR, c.T, F)) { failed = s + 1; break; }
     if (s == 0) Tacc = c.T;
     const double ha = h * c_ls_a[s], hb = h * c_ls_b[s], he = h * c_ls_e[s];
-    if constexpr (kMixed) {
-      const float ha_f = d2f(ha);
 #pragma unroll
-      for (int k = 0; k < NSP; ++k) {
-        U[k] = fmaf(ha_f, F[k], d2f(c.X[k]));
-        const double Fk = f2d(F[k]);
-        E[k] = fma(he, Fk, E[k]);
-        c.X[k] = fma(hb, Fk, c.X[k]);
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < NSP; ++k) {
-        E[k] = fma(he, F[k], E[k]);
-        U[k] = fma(ha, F[k], c.X[k]);
-        c.X[k] = fma(hb, F[k], c.X[k]);
-      }
+    for (int k = 0; k < NSP; ++k) {
+      E[k] = fma(he, F[k], E[k]);
+      U[k] = fma(ha, F[k], c.X[k]);
+      c.X[k] = fma(hb, F[k], c.X[k]);
     }
   }
   if (failed == 1) {
@@ -174,44 +185,93 @@ __device__ __forceinline__ void cell_attempt(const MechTables &mt, CellState &c,
     c.done = true;
     return;
   }
-  // WRMS norm; the weights' reciprocals are Newton-Raphson-refined (two steps, within
-  // 2 ulp, in the fp64 variant; one step, ~2^-40 relative, in the mixed one, whose fp32
-  // stages perturb the estimate far more)
-  double err = CUDART_NAN;
+  // WRMS norm; the weights' reciprocals are Newton-Raphson-refined (two steps, within 2 ulp)
+  double sum = CUDART_NAN;
   if (!failed) {
-    double sum = 0.0;
+    sum = 0.0;
 #pragma unroll
     for (int k = 0; k < NSP; ++k) {
-      const double den = fma(p.rtol, max_abs(Xs[k], c.X[k]), p.atol);
-      const double w = E[k] * (kMixed ? rcp1(den) : rcp2(den));
+      const double w = E[k] * rcp2(fma(p.rtol, max_abs(Xs[k], c.X[k]), p.atol));
       sum = fma(w, w, sum);
     }
-    err = sqrt(sum * (1.0 / NSP));
   }
   // a rejected attempt returns the cell to its accepted state, the temperature warm
   // start included (a trial stage's temperature can sit near another root of e(T) of the
   // extrapolated polynomials)
-  if (!isfinite(err)) {
+  if (!attempt_end(c, h, sum)) {
 #pragma unroll
     for (int k = 0; k < NSP; ++k) c.X[k] = Xs[k];
     c.T = Tacc;
-    ++c.nrej;
-    c.h = h * 0.2;
+  }
+}
+
+// One attempted step, mixed variant: the stage register U and F are fp32, X, the saved y_n
+// (c.X) and E fp64 (their updates cost 18 of the FP64 pipe's instructions a stage, in the
+// shadow of the right-hand side's FP32 work; the error sum cancels to ~1e-4 of its terms
+// and needs the 53 bits, and at the stability limit the scheme grows any perturbation of X).  The species loops stay rolled, as in rhs_mixed.cuh; c.X is then
+// indexed in local memory, four accesses a species and step.
+template <int ST>
+__device__ __forceinline__ void cell_attempt_mixed(const MechTables &mt, CellState &c, const StepParams &p) {
+  double h;
+  if (!attempt_begin(c, p, h)) return;
+  const MixedCols m = mixed_cols<ST>();
+  const ff eR = ff_norm(d2ff(c.eR));
+  ff T = ff_norm(d2ff(c.T)), Tacc = T;
+#pragma unroll 1
+  for (int k = 0; k < NSP; ++k) {
+    const double x = c.X[k];
+    m.X[k * ST] = x;
+    m.CU[k * ST].y = d2f(x);
+    m.E[k * ST] = 0.0;
+  }
+  int failed = 0;
+#pragma unroll 1
+  for (int s = 0; s < 5; ++s) {
+    ++c.nrhs;
+    if (!cell_rhs_mixed<ST>(mt, m, c.rho_f, c.invRho_f, eR, T)) { failed = s + 1; break; }
+    if (s == 0) Tacc = T;
+    const double ha = h * c_ls_a[s], hb = h * c_ls_b[s], he = h * c_ls_e[s];
+    const float ha_f = d2f(ha);
+#pragma unroll 3
+    for (int k = 0; k < NSP; ++k) {
+      const double x = m.X[k * ST];
+      const float f = m.Q[k * ST];
+      m.CU[k * ST].y = __fmaf_rn(ha_f, f, d2f(x));
+      const double fd = f2d(f);
+      m.E[k * ST] = fma(he, fd, m.E[k * ST]);
+      m.X[k * ST] = fma(hb, fd, x);
+    }
+  }
+  if (failed == 1) {
+    c.T = ff2d(T);
+    c.status = CHEM_CELL_NEWTON_FAIL;
+    c.done = true;
     return;
   }
-  // the step factor stays IEEE fp64: an explicit scheme at its stability limit grows a
-  // perturbation of h along its weakly unstable modes into another rejection sequence
-  const double fac = (err == 0.0) ? 5.0 : fmin(5.0, fmax(0.2, 0.9 / sqrt(sqrt(err))));
-  if (err <= 1.0) {
-    c.t += h;
-    ++c.nacc;
-  } else {
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) c.X[k] = Xs[k];
-    c.T = Tacc;
-    ++c.nrej;
+  // WRMS norm in fp64; the weights' reciprocals take one Newton-Raphson step (~2^-40
+  // relative; the fp32 stages perturb the estimate far more)
+  double sum = CUDART_NAN;
+  if (!failed) {
+    sum = 0.0;
+#pragma unroll 1
+    for (int k = 0; k < NSP; ++k) {
+      const double w = m.E[k * ST] * rcp1(fma(p.rtol, max_abs(c.X[k], m.X[k * ST]), p.atol));
+      sum = fma(w, w, sum);
+    }
   }
-  c.h = h * fac;
+  if (attempt_end(c, h, sum)) {
+#pragma unroll 1
+    for (int k = 0; k < NSP; ++k) c.X[k] = m.X[k * ST];
+    c.T = ff2d(T);
+  } else {  // back to the accepted state and its temperature, as in fp64
+    c.T = ff2d(Tacc);
+  }
+}
+
+template <int V, int BLOCK>
+__device__ __forceinline__ void cell_attempt(const MechTables &mt, CellState &c, const StepParams &p) {
+  if constexpr (V == CHEM_VARIANT_MIXED) cell_attempt_mixed<BLOCK>(mt, c, p);
+  else cell_attempt_fp64(mt, c, p);
 }
 
 // One attempted step of a full-storage scheme (CHEM_SCHEME_FULL_STORAGE: table 0, five
@@ -220,7 +280,7 @@ __device__ __forceinline__ void cell_attempt(const MechTables &mt, CellState &c,
 // side is inlined once); the stage derivatives live in a register array indexed by
 // compile-time constants, written through predicated moves, so the k-storage costs
 // registers (and spills), not local-memory indexing.
-template <int V, int SCH>
+template <int V, int SCH, int BLOCK>
 __device__ __forceinline__ void cell_attempt_full(const MechTables &mt, CellState &c,
                                                   const StepParams &p) {
   constexpr bool kMixed = V == CHEM_VARIANT_MIXED;
@@ -240,6 +300,11 @@ __device__ __forceinline__ void cell_attempt_full(const MechTables &mt, CellStat
     for (int k = 0; k < NSP; ++k) K[j][k] = SReal(0);
   int failed = 0;
   double Tacc = c.T;
+  ff Tf{}, eRf{};
+  if constexpr (kMixed) {
+    Tf = ff_norm(d2ff(c.T));
+    eRf = ff_norm(d2ff(c.eR));
+  }
 #pragma unroll 1
   for (int s = 0; s < S; ++s) {
     SReal U[NSP], F[NSP];
@@ -261,8 +326,17 @@ __device__ __forceinline__ void cell_attempt_full(const MechTables &mt, CellStat
     }
     ++c.nrhs;
     bool ok;
-    if constexpr (kMixed) ok = cell_rhs_mixed(mt, U, c.rho_f, c.invRho_f, c.eR, c.T, F);
-    else ok = cell_rhs(mt, U, c.rho, c.invRho, c.eR, c.T, F);
+    if constexpr (kMixed) {
+      const MixedCols m = mixed_cols<BLOCK>();
+#pragma unroll
+      for (int k = 0; k < NSP; ++k) m.CU[k * BLOCK].y = U[k];
+      ok = cell_rhs_mixed<BLOCK>(mt, m, c.rho_f, c.invRho_f, eRf, Tf);
+#pragma unroll
+      for (int k = 0; k < NSP; ++k) F[k] = m.Q[k * BLOCK];
+      c.T = ff2d(Tf);
+    } else {
+      ok = cell_rhs(mt, U, c.rho, c.invRho, c.eR, c.T, F);
+    }
     if (!ok) { failed = s + 1; break; }
     if (s == 0) Tacc = c.T;
 #pragma unroll

@@ -92,14 +92,15 @@ __device__ __forceinline__ void store_ln_inv_kc(const Gibbs &g, double *o, std::
 // temperature solve), form 1 the error test's all-fp32 one.
 __global__ void k_ln_inv_kc(const __grid_constant__ MechTables mt, int form, int64_t n,
                             const double *__restrict__ T, double *__restrict__ out) {
-  load_math_tables();  // log_t reads the per-block tables
+  load_mixed_tables<1>(mt);
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double t = T[i];
   double *o = out + i * NRX;
   if (form == 0) {
     GibbsHL g;
-    gibbs_hl(mt, t, log_t(t), rcp1(t), g);
+    const ff tf = ff_norm(d2ff(t));
+    gibbs_hl<1>(mt, tf, ff_log(tf), d2ff(rcp1(t)), g.g, g.r);
     store_ln_inv_kc(g, o, std::make_integer_sequence<int, NRX>{});
   } else {
     const float tf = (float)t;

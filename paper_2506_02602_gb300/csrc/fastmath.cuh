@@ -69,14 +69,10 @@ static __device__ __noinline__ double exp_t(double x) {
   return fma(ts, p, ts);
 }
 
-// log(x) for positive normal finite x (the kernels' arguments: temperatures, F_cent,
-// Pr); zero, subnormal, negative, inf and NaN inputs fall back to the library log via
-// an integer test of the exponent field.
-__device__ __forceinline__ double log_t(double x) {
+// log(x) for positive normal finite x.
+__device__ __forceinline__ double log_tab(double x) {
   const long long bits = __double_as_longlong(x);
-  const int ef = (int)(bits >> 52);  // sign and biased exponent
-  if (ef <= 0 || ef >= 0x7ff) return log(x);
-  const int ex = ef - 1023;
+  const int ex = (int)(bits >> 52) - 1023;
   const long long mb = bits & 0x000fffffffffffffLL;
   const int j = (int)(((mb >> 45) + 1) >> 1);  // nearest 64th of the fraction, 0..64
   const double f = __longlong_as_double(mb | 0x3ff0000000000000LL);
@@ -93,6 +89,14 @@ __device__ __forceinline__ double log_t(double x) {
   if (ex == -1) return s_log_tab_m1[j] + l1p;
   const double e = (double)ex;
   return fma(e, kLn2Hi, s_log_tab[j] + fma(e, kLn2Lo, l1p));
+}
+
+// log(x) of the kernels' arguments (temperatures, F_cent, Pr); zero, subnormal, negative, inf
+// and NaN inputs fall back to the library log via an integer test of the exponent field.
+__device__ __forceinline__ double log_t(double x) {
+  const int ef = (int)(__double_as_longlong(x) >> 52);  // sign and biased exponent
+  if (ef <= 0 || ef >= 0x7ff) return log(x);
+  return log_tab(x);
 }
 
 __device__ __forceinline__ double log10_t(double x) { return log_t(x) * kInvLn10; }
@@ -186,9 +190,21 @@ __device__ __forceinline__ double clamp_abs(double x, double lim) {
 // whose magnitude stays below 2^12 is exact in fp32, so an fp64 sum with heavy
 // cancellation (ln K_c from Gibbs functions of magnitude up to a few hundred) is
 // assembled in fp32 to within an ulp of the result plus ~1e-11.
+// In that range the fraction bits below the grid are an integer of up to 52 bits, whose
+// conversion to fp32 rounds as x - hi would: no FP64 instruction.
 __device__ __forceinline__ void split_hilo(double x, float &hi, float &lo) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int n = 40 - ((int)((b >> 52) & 0x7ff) - 1023);  // fraction bits worth < 2^-12
+  const int ex = (int)((b >> 52) & 0x7ff);
+  const int n = 1063 - ex;  // fraction bits worth < 2^-12
+  if ((unsigned)(n - 29) < 24u) {  // 2^-12 <= |x| < 2^12
+    const uint32_t h = (uint32_t)(b >> 32);
+    const unsigned long long low = b & ~(~0ull << n), top = b ^ low;
+    const uint32_t t = (uint32_t)(top >> 29) - 0xc0000000u;  // exponent bias 1023 -> 127; 24 bits at most, exact
+    hi = __uint_as_float((t & 0x7fffffffu) | (h & 0x80000000u));
+    const float l = (float)(long long)low * __uint_as_float((uint32_t)(ex - 948) << 23);
+    lo = __uint_as_float(__float_as_uint(l) | (h & 0x80000000u));
+    return;
+  }
   const unsigned long long mask = n >= 53 ? 0ull : (n <= 0 ? ~0ull : (~0ull << n));
   const double h = __longlong_as_double((long long)(b & mask));
   hi = d2f(h);

@@ -10,10 +10,14 @@ f in [1, 2), c_j = RN(1 / (1 + j/64)) with j the nearest 64th of f - 1, r = f c_
 stored double c_j.  For inputs in [0.5, 1) (e = -1) a second table holds -ln(2 c_j), so
 the result near 1 keeps full relative accuracy.
 
+Double-float log (ff.cuh): the same reduction with c_j rounded to fp32, -ln(c_j) of the stored
+c_j as a pair of fp32 numbers, and ln2 as a 16-bit number plus a pair.
+
 Every value is computed with 60-digit decimal arithmetic and rounded once to double.
 Run:  python gen_math_tables.py > math_tables.cuh
 """
 from decimal import Decimal, getcontext
+from struct import pack, unpack
 
 getcontext().prec = 60
 LN2 = Decimal(2).ln()
@@ -21,6 +25,15 @@ LN2 = Decimal(2).ln()
 
 def hexd(x: Decimal) -> str:
     return float(x).hex()
+
+
+def f32(x) -> float:
+    return unpack("f", pack("f", float(x)))[0]
+
+
+def pair(x: Decimal):
+    h = f32(x)
+    return h, f32(x - Decimal(h))
 
 
 def main():
@@ -48,13 +61,23 @@ def main():
     for c in inv:
         out.append(f"    {hexd(-(2 * Decimal(c)).ln())},")
     out.append("};")
+    out.append("// {c_j = RN32(1 / (1 + j/64)), -ln(c_j) as a pair, 0}, j = 0..64")
+    out.append("__device__ const float k_ln_ff[65][4] = {")
+    for j in range(65):
+        c = f32(1 / (1 + Decimal(j) / 64))
+        h, lo = pair(-Decimal(c).ln())
+        out.append(f"    {{{c.hex()}f, {h.hex()}f, {lo.hex()}f, 0.0f}},")
+    out.append("};")
     ln2 = float(LN2)
+    ln2a = 0.693145751953125
+    ln2b, ln2c = pair(LN2 - Decimal(ln2a))
     out += [
         f"constexpr double kLn2Hi = {ln2.hex()};",
         f"constexpr double kLn2Lo = {hexd(LN2 - Decimal(ln2))};",
         f"constexpr double kInvLn2x128 = {hexd(128 / LN2)};",
         f"constexpr double kLn2d128Hi = {float(LN2 / 128).hex()};",
         f"constexpr double kLn2d128Lo = {hexd(LN2 / 128 - Decimal(float(LN2 / 128)))};",
+        f"constexpr float kLn2A = {ln2a.hex()}f, kLn2B = {ln2b.hex()}f, kLn2C = {ln2c.hex()}f;",
         f"constexpr double kLn10 = {hexd(Decimal(10).ln())};",
         f"constexpr double kInvLn10 = {hexd(1 / Decimal(10).ln())};",
         "", "}  // namespace chem", ""]

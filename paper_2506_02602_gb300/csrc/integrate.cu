@@ -9,14 +9,19 @@ namespace chem {
 
 // BLOCK threads per block, MINB resident blocks per SM.  The register file is split
 // between the SM's four sub-partitions, so 12 warps per SM allow 170 registers a thread
-// (128 x 3), 16 warps 128 (64 x 8, 32 x 16) and 32 warps 64 (64 x 16, 32 x 32); anything
-// between rounds down; 8 warps (256 x 1) leave the 255-register maximum.
+// (128 x 3), 16 warps 128 (64 x 8, 32 x 16, 128 x 4) and 32 warps 64 (64 x 16, 32 x 32);
+// anything between rounds down; 8 warps (256 x 1) leave the 255-register maximum.
 // SCH: CHEM_SCHEME_LSRK (the two-register scheme of Eq. 21) or one of the full-storage
 // comparators (cell_attempt_full).
 template <int V, int BLOCK, int MINB, int SCH = CHEM_SCHEME_LSRK>
 __global__ void __launch_bounds__(BLOCK, MINB) k_lsrk(const __grid_constant__ MechTables mt,
                                                       const CellArgs a, const StepParams p) {
-  load_math_tables();
+  if constexpr (V == CHEM_VARIANT_MIXED) {
+    load_mixed_tables<BLOCK>(mt);
+    init_mixed_cols<BLOCK>(mixed_cols<BLOCK>());
+  } else {
+    load_math_tables();
+  }
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool live = i < a.n;
   CellState c;
@@ -29,9 +34,9 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_lsrk(const __grid_constant__ Me
     c.h = a.h ? a.h[i] : CUDART_NAN;
     cell_begin(c, a.rho[i], a.e[i], p.dt);
     if constexpr (SCH == CHEM_SCHEME_LSRK) {
-      while (!c.done) cell_attempt<V>(mt, c, p);
+      while (!c.done) cell_attempt<V, BLOCK>(mt, c, p);
     } else {
-      while (!c.done) cell_attempt_full<V, SCH>(mt, c, p);
+      while (!c.done) cell_attempt_full<V, SCH, BLOCK>(mt, c, p);
     }
     cell_finish(mt, c);
 #pragma unroll
@@ -68,43 +73,48 @@ __global__ void k_state_from_TPY(const __grid_constant__ MechTables mt, int64_t 
   e[i] = R_U * e_over_R(m, Ti);
 }
 
-// Blocks per SM of the 32- and 64-thread shapes.  The mixed two-register kernel runs them
-// at 32 warps per SM (64 registers, spilling to L1 and L2): the FP64 pipe's latency is
-// hidden by more warps rather than by registers, and the 1M-cell detonation slice ran
-// 3.8 % faster than at 16 warps (128 registers) with the 9-species structure, 4.3 % with
-// the 13-species one.  The fp64 variant (fp64 state and rates) and the full-storage
-// comparators keep 16 warps: the fp64 kernel measured 7 % slower at 32.
-template <int V, int SCH>
-constexpr int kDense = (V == CHEM_VARIANT_MIXED && SCH == CHEM_SCHEME_LSRK) ? 2 : 1;
+// Launch with the mixed variant's dynamic shared memory (the per-thread columns).
+template <int V, int BLOCK, int MINB, int SCH>
+static cudaError_t launch_one(const MechTables &mt, const CellArgs &a, const StepParams &p, cudaStream_t s) {
+  size_t smem = 0;
+  if constexpr (V == CHEM_VARIANT_MIXED) {
+    smem = mixed_cols_bytes(BLOCK);
+    const cudaError_t e = allow_smem(reinterpret_cast<const void *>(k_lsrk<V, BLOCK, MINB, SCH>), smem);
+    if (e != cudaSuccess) return e;
+  }
+  k_lsrk<V, BLOCK, MINB, SCH><<<(unsigned)((a.n + BLOCK - 1) / BLOCK), BLOCK, smem, s>>>(mt, a, p);
+  return cudaGetLastError();
+}
 
+// The compiled shapes.  fp64: 12 warps per SM (128 x 3, 166 registers, no spills) or 16 (32, 64
+// threads, 128 registers).  The mixed two-register kernel's per-thread columns allow 16 warps
+// per SM (12 with 13 species): 128 x 4 at 128 registers, 7.9 ms on the 1M-cell detonation slice;
+// its 32- and 64-thread shapes keep 64 registers (14 warps of 64 threads, spilling): 9.3 ms at
+// 64, 11.2 at 32.
 template <int V, int SCH>
-static void launch_shape(const MechTables &mt, const CellArgs &a, const StepParams &p, int block,
-                         cudaStream_t s) {
-  const unsigned grid = (unsigned)((a.n + block - 1) / block);
-  if (block == 32) k_lsrk<V, 32, 16 * kDense<V, SCH>, SCH><<<grid, 32, 0, s>>>(mt, a, p);
-  else if (block == 64) k_lsrk<V, 64, 8 * kDense<V, SCH>, SCH><<<grid, 64, 0, s>>>(mt, a, p);
-  else if (block == 256) k_lsrk<V, 256, 1, SCH><<<grid, 256, 0, s>>>(mt, a, p);
-  else k_lsrk<V, 128, 3, SCH><<<grid, 128, 0, s>>>(mt, a, p);
+static cudaError_t launch_shape(const MechTables &mt, const CellArgs &a, const StepParams &p, int block,
+                                cudaStream_t s) {
+  constexpr bool dense = V == CHEM_VARIANT_MIXED && SCH == CHEM_SCHEME_LSRK;
+  if (block == 32) return launch_one<V, 32, dense ? 32 : 16, SCH>(mt, a, p, s);
+  if (block == 64) return launch_one<V, 64, dense ? 16 : 8, SCH>(mt, a, p, s);
+  if (block == 256) return launch_one<V, 256, 1, SCH>(mt, a, p, s);
+  return launch_one<V, 128, dense && NSP <= 9 ? 4 : 3, SCH>(mt, a, p, s);
 }
 
 template <int SCH>
-static void launch_variant(int variant, const MechTables &mt, const CellArgs &a,
-                           const StepParams &p, int block, cudaStream_t s) {
-  if (variant == CHEM_VARIANT_MIXED) launch_shape<CHEM_VARIANT_MIXED, SCH>(mt, a, p, block, s);
-  else launch_shape<CHEM_VARIANT_FP64, SCH>(mt, a, p, block, s);
+static cudaError_t launch_variant(int variant, const MechTables &mt, const CellArgs &a,
+                                  const StepParams &p, int block, cudaStream_t s) {
+  if (variant == CHEM_VARIANT_MIXED) return launch_shape<CHEM_VARIANT_MIXED, SCH>(mt, a, p, block, s);
+  return launch_shape<CHEM_VARIANT_FP64, SCH>(mt, a, p, block, s);
 }
 
 cudaError_t launch_lsrk(int variant, int scheme, const MechTables &mt, const CellArgs &a,
                         const StepParams &p, int block, cudaStream_t s) {
   if (a.n <= 0) return cudaSuccess;
-  if (block != 32 && block != 64 && block != 256) block = 128;  // the compiled shapes
   if (scheme == CHEM_SCHEME_FULL_STORAGE)
-    launch_variant<CHEM_SCHEME_FULL_STORAGE>(variant, mt, a, p, block, s);
-  else if (scheme == CHEM_SCHEME_RKF45)
-    launch_variant<CHEM_SCHEME_RKF45>(variant, mt, a, p, block, s);
-  else
-    launch_variant<CHEM_SCHEME_LSRK>(variant, mt, a, p, block, s);
-  return cudaGetLastError();
+    return launch_variant<CHEM_SCHEME_FULL_STORAGE>(variant, mt, a, p, block, s);
+  if (scheme == CHEM_SCHEME_RKF45) return launch_variant<CHEM_SCHEME_RKF45>(variant, mt, a, p, block, s);
+  return launch_variant<CHEM_SCHEME_LSRK>(variant, mt, a, p, block, s);
 }
 
 cudaError_t launch_state_from_TPY(const MechTables &mt, int64_t n, const double *T,

@@ -64,6 +64,13 @@ struct BatchScratch {
   unsigned long long *cursor;    // [1] next queue slot
 };
 
+// Lets kernel fn use `bytes` of dynamic shared memory on the current device (needed above
+// 48 KB; set before each launch, as the setting is per device).
+inline cudaError_t allow_smem(const void *fn, size_t bytes) {
+  return bytes <= 40 * 1024 ? cudaSuccess
+                            : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 // Launchers (integrate.cu).  Return the cudaError_t of the launch.
 cudaError_t launch_lsrk(int variant, int scheme, const MechTables &mt, const CellArgs &a,
                         const StepParams &p, int block, cudaStream_t s);
@@ -90,8 +97,7 @@ cudaError_t launch_batched(int variant, const MechTables &mt, const BatchArgs &a
                            const StepParams &p, const BatchScratch &s, int order_mode,
                            int ctas_per_sm, int shape, cudaStream_t st);
 // The persistent kernel over a given queue of cell indices (order[0 .. queue length))
-// with the variant's fastest shape (0 for fp64, the 32-warp shape 4 for mixed) and all
-// resident CTAs; resets the cursor first.
+// with the default shape (the fastest of each variant) and all resident CTAs; resets the cursor first.
 cudaError_t launch_persistent_queue(int variant, const MechTables &mt, const BatchArgs &a,
                                     const StepParams &p, const int32_t *order,
                                     unsigned long long *cursor, cudaStream_t st);

@@ -59,6 +59,11 @@ struct MechTablesF32 {
   float gc[2][NSP][7];
   float T_mid, ln_R_over_Pref;
   float newton_sq;  // the fp64 Newton's stop constant (below), tested in fp32
+  // fp32 pairs (value = [0] + [1] to ~2^-49) of ecw, gc, T_mid and ln_R_over_Pref below,
+  // for the mixed right-hand side's double-float arithmetic (ff.cuh)
+  float ecw2[2][NSP][6][2];
+  float gc2[2][NSP][7][2];
+  float T_mid2[2], ln_R_over_Pref2[2];
 };
 
 // Per-context tables (host-built from chem_mechanism by build_tables()).
