@@ -111,59 +111,44 @@ __device__ __forceinline__ bool solve_T(const MechTables &mt, const double (&Y)[
 // Quantities shared by every reaction of one evaluation.
 struct RateInputs {
   double lnT, invT, RTP, PRT, ctot;
-  long long lT, iT;  // log2 T (Q58), 1 / T (Q70): the fixed-point form's
-  double c[NSP];     // clamped concentrations, mol/m^3
-  double G[NSP];     // exp(-g_k / (R_u T))
-  double iG[NSP];    // c_k / G_k
+  double c[NSP];   // clamped concentrations, mol/m^3
+  double G[NSP];   // exp(-g_k / (R_u T))
+  double iG[NSP];  // 1 / G_k (with the one-way fluxes) or c_k / G_k (net rates only)
 };
 
-// Temperatures of the fixed-point form: (128, 32768), on the high word.
-__device__ __forceinline__ bool fixed_range(double T) {
-  return (uint32_t)__double2hiint(T) - 0x40600001u < 0x40e00000u - 0x40600001u;
-}
-
 // Troe broadening factor (Gilbert, Luther & Troe 1983).
-template <int J, bool kFixed>
+template <int J>
 __device__ __forceinline__ double troe_F(const MechTables &mt, double T, double invT, double Pr) {
   constexpr int n = kRx[J].troe_n;
   if constexpr (n == 0) {
     return 1.0;
   } else {
     const double a = mt.troe_a[J];
-    double Fc;
-    if constexpr (kFixed) {
-      Fc = (1.0 - a) * exp2_lim(-T * mt.troe_q3[J]) + a * exp2_lim(-T * mt.troe_q1[J]);
-      if constexpr (n == 4) Fc += exp2_lim(-mt.troe_q2[J] * invT);
-    } else {
-      Fc = (1.0 - a) * exp_t(-T * mt.troe_i3[J]) + a * exp_t(-T * mt.troe_i1[J]);
-      if constexpr (n == 4) Fc += exp_t(-mt.troe_T2[J] * invT);
-    }
+    double Fc = (1.0 - a) * exp_t(-T * mt.troe_i3[J]) + a * exp_t(-T * mt.troe_i1[J]);
+    if constexpr (n == 4) Fc += exp_t(-mt.troe_T2[J] * invT);
     const double lFc = log10_t(Fc);
     const double cc = -0.4 - 0.67 * lFc;
     const double nn = 0.75 - 1.27 * lFc;
     const double x = log10_t(Pr) + cc;
     const double f1 = x * rcp2(nn - 0.14 * x);
-    const double lF = lFc * rcp2(1.0 + f1 * f1);
-    if constexpr (kFixed) return exp2_lim(lF * kLog2_10);
-    else return exp10_t(lF);
+    return exp10_t(lFc / (1.0 + f1 * f1));
   }
 }
 
-// Rate of progress of reaction J added into wdot (law of mass action, Eq. 16).  kFixed: the
-// exponentials in fixed point.
-template <int J, bool kFixed>
+// Rate of progress of reaction J added into wdot (law of mass action, Eq. 16).  With
+// kDestr, the one-way fluxes that consume each species are also summed into dflux
+// (used by the stiffness probe: consumption rate per unit concentration).
+template <int J, bool kDestr = false>
 __device__ __forceinline__ void reaction(const MechTables &mt, const RateInputs &in, double T,
-                                         double (&wdot)[NSP]) {
+                                         double (&wdot)[NSP], double *dflux = nullptr) {
   constexpr RxStruct R = kRx[J];
   constexpr int dnu = n_prod(R) - n_reac(R);
   static_assert(dnu >= -1 && dnu <= 1, "compiled structure assumes |sum nu| <= 1");
   // kconst: 0 Arrhenius exponential; 1 constant (b = Ea = 0); 2, 3: A T^-1, A T^-2 (Ea = 0)
   const int kc = mt.kconst[J];
   double kf;
-  if (kc == 0) {
-    if constexpr (kFixed) kf = exp2_q52(limit_q52(arrhenius_log2(mt.qA[J], mt.qB[J], mt.qH[J], in.lT, in.iT)));
-    else kf = exp_t(fma(mt.beta[J], in.lnT, mt.lnA[J]) - mt.Ta[J] * in.invT);
-  } else if (kc == 1) kf = mt.A[J];
+  if (kc == 0) kf = exp_t(fma(mt.beta[J], in.lnT, mt.lnA[J]) - mt.Ta[J] * in.invT);
+  else if (kc == 1) kf = mt.A[J];
   else if (kc == 2) kf = mt.A[J] * in.invT;
   else kf = mt.A[J] * in.invT * in.invT;
   double M = 0.0;
@@ -176,26 +161,48 @@ __device__ __forceinline__ void reaction(const MechTables &mt, const RateInputs 
     }
   }
   if constexpr (R.type == FALLOFF) {
-    double k0;
-    if constexpr (kFixed) k0 = exp2_q52(limit_q52(arrhenius_log2(mt.qA0[J], mt.qB0[J], mt.qH0[J], in.lT, in.iT)));
-    else k0 = exp_t(fma(mt.beta0[J], in.lnT, mt.lnA0[J]) - mt.Ta0[J] * in.invT);
+    const double k0 = exp_t(fma(mt.beta0[J], in.lnT, mt.lnA0[J]) - mt.Ta0[J] * in.invT);
     const double Pr = k0 * M * rcp2(kf);
-    kf = (Pr > 0.0) ? kf * (Pr * rcp2(1.0 + Pr)) * troe_F<J, kFixed>(mt, T, in.invT, Pr) : 0.0;
+    kf = (Pr > 0.0) ? kf * (Pr * rcp2(1.0 + Pr)) * troe_F<J>(mt, T, in.invT, Pr) : 0.0;
   }
-  // q = k_f (prod c_reactants - prod G_reactants prod (c / G)_products (R_u T / p)^dnu),
-  // the same net rate as k_f prod c - k_r prod c with k_r = k_f / K_c
-  double cf = in.c[R.r0];
-  if constexpr (R.r1 >= 0) cf *= in.c[R.r1];
-  if (mt.reversible[J]) {
-    double gr = in.G[R.r0];
-    if constexpr (R.r1 >= 0) gr *= in.G[R.r1];
-    if constexpr (dnu == 1) gr *= in.RTP;
-    if constexpr (dnu == -1) gr *= in.PRT;
-    double ap = in.iG[R.p0];
-    if constexpr (R.p1 >= 0) ap *= in.iG[R.p1];
-    cf = fma(-gr, ap, cf);
+  double q;
+  if constexpr (kDestr) {
+    double qf = kf * in.c[R.r0];
+    if constexpr (R.r1 >= 0) qf *= in.c[R.r1];
+    double qr = 0.0;
+    q = qf;
+    if (mt.reversible[J]) {
+      double kr = kf * in.G[R.r0];
+      if constexpr (R.r1 >= 0) kr *= in.G[R.r1];
+      kr *= in.iG[R.p0];
+      if constexpr (R.p1 >= 0) kr *= in.iG[R.p1];
+      if constexpr (dnu == 1) kr *= in.RTP;
+      if constexpr (dnu == -1) kr *= in.PRT;
+      qr = kr * in.c[R.p0];
+      if constexpr (R.p1 >= 0) qr *= in.c[R.p1];
+      q = qf - qr;
+    }
+    const double m = (R.type == THIRD_BODY) ? M : 1.0;
+    dflux[R.r0] += m * qf;
+    if constexpr (R.r1 >= 0) dflux[R.r1] += m * qf;
+    dflux[R.p0] += m * qr;
+    if constexpr (R.p1 >= 0) dflux[R.p1] += m * qr;
+  } else {
+    // q = k_f (prod c_reactants - prod G_reactants prod (c / G)_products (R_u T / p)^dnu),
+    // the same net rate as k_f prod c - k_r prod c with k_r = k_f / K_c
+    double cf = in.c[R.r0];
+    if constexpr (R.r1 >= 0) cf *= in.c[R.r1];
+    if (mt.reversible[J]) {
+      double gr = in.G[R.r0];
+      if constexpr (R.r1 >= 0) gr *= in.G[R.r1];
+      if constexpr (dnu == 1) gr *= in.RTP;
+      if constexpr (dnu == -1) gr *= in.PRT;
+      double ap = in.iG[R.p0];
+      if constexpr (R.p1 >= 0) ap *= in.iG[R.p1];
+      cf = fma(-gr, ap, cf);
+    }
+    q = kf * cf;
   }
-  double q = kf * cf;
   if constexpr (R.type == THIRD_BODY) q *= M;
   wdot[R.r0] -= q;
   if constexpr (R.r1 >= 0) wdot[R.r1] -= q;
@@ -203,25 +210,24 @@ __device__ __forceinline__ void reaction(const MechTables &mt, const RateInputs 
   if constexpr (R.p1 >= 0) wdot[R.p1] += q;
 }
 
-template <bool kFixed, int... J>
+template <bool kDestr, int... J>
 __device__ __forceinline__ void all_reactions(const MechTables &mt, const RateInputs &in, double T,
-                                              double (&wdot)[NSP], std::integer_sequence<int, J...>) {
-  (reaction<J, kFixed>(mt, in, T, wdot), ...);
+                                              double (&wdot)[NSP], double *dflux,
+                                              std::integer_sequence<int, J...>) {
+  (reaction<J, kDestr>(mt, in, T, wdot, dflux), ...);
 }
 
 // Molar production rates wdot (mol/m^3/s) at temperature T and clamped concentrations c.
-template <bool kFixed>
+// kDestr: also the consumption fluxes per species into dflux (zeroed here).
+template <bool kDestr = false>
 __device__ __forceinline__ void production_rates(const MechTables &mt, double T,
-                                                 const double (&c)[NSP], double (&wdot)[NSP]) {
+                                                 const double (&c)[NSP], double (&wdot)[NSP],
+                                                 double *dflux = nullptr) {
   RateInputs in;
   in.lnT = log_t(T);
   in.invT = rcp2(T);
   in.RTP = (R_U / P_REF) * T;
   in.PRT = (P_REF / R_U) * in.invT;
-  if constexpr (kFixed) {
-    in.lT = (long long)abs_q<58>(in.lnT * kLog2E);
-    in.iT = (long long)abs_q<70>(in.invT);
-  }
   const double oml = 1.0 - in.lnT;
   const int range = ge_nonneg(T, mt.T_mid);
   double ctot = 0.0;
@@ -229,35 +235,18 @@ __device__ __forceinline__ void production_rates(const MechTables &mt, double T,
   for (int k = 0; k < NSP; ++k) {
     in.c[k] = c[k];
     ctot += c[k];
-    const double *gc = kFixed ? mt.gc_q[range][k] : mt.gc[range][k];
+    const double *gc = mt.gc[range][k];
     double g = fma(T, fma(T, fma(T, fma(T, gc[4], gc[3]), gc[2]), gc[1]), fma(gc[5], in.invT, gc[6]));
     g = fma(gc[0], oml, g);
-    // the limits keep G finite far outside the tables' range
-    if constexpr (kFixed) {
-      const long long y = to_q52(g);
-      in.G[k] = exp2_q52(y);
-      in.iG[k] = c[k] * exp2_q52(-y);
-    } else {
-      g = clamp_abs(g, 700.0);
-      in.G[k] = exp_t(-g);
-      in.iG[k] = c[k] * rcp2(in.G[k]);
-    }
+    // clamp keeps G finite far outside the tables' range
+    g = clamp_abs(g, 700.0);
+    in.G[k] = exp_t(-g);
+    in.iG[k] = kDestr ? rcp2(in.G[k]) : c[k] * rcp2(in.G[k]);
     wdot[k] = 0.0;
+    if constexpr (kDestr) dflux[k] = 0.0;
   }
   in.ctot = ctot;
-  all_reactions<kFixed>(mt, in, T, wdot, std::make_integer_sequence<int, NRX>{});
-}
-
-// The form on exp_t, for temperatures or coefficients outside the fixed-point form's range;
-// out of line, as few evaluations come here.
-static __device__ __noinline__ void production_rates_any(const MechTables &mt, double T, const double *c,
-                                                         double *wdot) {
-  double cc[NSP], w[NSP];
-#pragma unroll
-  for (int k = 0; k < NSP; ++k) cc[k] = c[k];
-  production_rates<false>(mt, T, cc, w);
-#pragma unroll
-  for (int k = 0; k < NSP; ++k) wdot[k] = w[k];
+  all_reactions<kDestr>(mt, in, T, wdot, dflux, std::make_integer_sequence<int, NRX>{});
 }
 
 // dY/dt of one cell at fixed (rho, e).  T: in = Newton guess, out = solved T.
@@ -268,16 +257,7 @@ __device__ __forceinline__ bool cell_rhs(const MechTables &mt, const double (&Y)
   double c[NSP], wdot[NSP];
 #pragma unroll
   for (int k = 0; k < NSP; ++k) c[k] = clamp_nonneg(rho * (Y[k] * mt.invW[k]));
-  if (mt.fixed_ok && fixed_range(T)) {
-    production_rates<true>(mt, T, c, wdot);
-  } else {
-    double cc[NSP], w[NSP];
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) cc[k] = c[k];
-    production_rates_any(mt, T, cc, w);
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) wdot[k] = w[k];
-  }
+  production_rates(mt, T, c, wdot);
 #pragma unroll
   for (int k = 0; k < NSP; ++k) F[k] = wdot[k] * mt.W[k] * invRho;
   return true;
