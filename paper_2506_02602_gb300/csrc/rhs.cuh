@@ -113,7 +113,7 @@ struct RateInputs {
   double lnT, invT, RTP, PRT, ctot;
   double c[NSP];   // clamped concentrations, mol/m^3
   double G[NSP];   // exp(-g_k / (R_u T))
-  double iG[NSP];  // 1 / G_k (with the one-way fluxes) or c_k / G_k (net rates only)
+  double iG[NSP];  // c_k / G_k
 };
 
 // Troe broadening factor (Gilbert, Luther & Troe 1983).
@@ -135,12 +135,10 @@ __device__ __forceinline__ double troe_F(const MechTables &mt, double T, double 
   }
 }
 
-// Rate of progress of reaction J added into wdot (law of mass action, Eq. 16).  With
-// kDestr, the one-way fluxes that consume each species are also summed into dflux
-// (used by the stiffness probe: consumption rate per unit concentration).
-template <int J, bool kDestr = false>
+// Rate of progress of reaction J added into wdot (law of mass action, Eq. 16).
+template <int J>
 __device__ __forceinline__ void reaction(const MechTables &mt, const RateInputs &in, double T,
-                                         double (&wdot)[NSP], double *dflux = nullptr) {
+                                         double (&wdot)[NSP]) {
   constexpr RxStruct R = kRx[J];
   constexpr int dnu = n_prod(R) - n_reac(R);
   static_assert(dnu >= -1 && dnu <= 1, "compiled structure assumes |sum nu| <= 1");
@@ -165,44 +163,20 @@ __device__ __forceinline__ void reaction(const MechTables &mt, const RateInputs 
     const double Pr = k0 * M * rcp2(kf);
     kf = (Pr > 0.0) ? kf * (Pr * rcp2(1.0 + Pr)) * troe_F<J>(mt, T, in.invT, Pr) : 0.0;
   }
-  double q;
-  if constexpr (kDestr) {
-    double qf = kf * in.c[R.r0];
-    if constexpr (R.r1 >= 0) qf *= in.c[R.r1];
-    double qr = 0.0;
-    q = qf;
-    if (mt.reversible[J]) {
-      double kr = kf * in.G[R.r0];
-      if constexpr (R.r1 >= 0) kr *= in.G[R.r1];
-      kr *= in.iG[R.p0];
-      if constexpr (R.p1 >= 0) kr *= in.iG[R.p1];
-      if constexpr (dnu == 1) kr *= in.RTP;
-      if constexpr (dnu == -1) kr *= in.PRT;
-      qr = kr * in.c[R.p0];
-      if constexpr (R.p1 >= 0) qr *= in.c[R.p1];
-      q = qf - qr;
-    }
-    const double m = (R.type == THIRD_BODY) ? M : 1.0;
-    dflux[R.r0] += m * qf;
-    if constexpr (R.r1 >= 0) dflux[R.r1] += m * qf;
-    dflux[R.p0] += m * qr;
-    if constexpr (R.p1 >= 0) dflux[R.p1] += m * qr;
-  } else {
-    // q = k_f (prod c_reactants - prod G_reactants prod (c / G)_products (R_u T / p)^dnu),
-    // the same net rate as k_f prod c - k_r prod c with k_r = k_f / K_c
-    double cf = in.c[R.r0];
-    if constexpr (R.r1 >= 0) cf *= in.c[R.r1];
-    if (mt.reversible[J]) {
-      double gr = in.G[R.r0];
-      if constexpr (R.r1 >= 0) gr *= in.G[R.r1];
-      if constexpr (dnu == 1) gr *= in.RTP;
-      if constexpr (dnu == -1) gr *= in.PRT;
-      double ap = in.iG[R.p0];
-      if constexpr (R.p1 >= 0) ap *= in.iG[R.p1];
-      cf = fma(-gr, ap, cf);
-    }
-    q = kf * cf;
+  // q = k_f (prod c_reactants - prod G_reactants prod (c / G)_products (R_u T / p)^dnu),
+  // the same net rate as k_f prod c - k_r prod c with k_r = k_f / K_c
+  double cf = in.c[R.r0];
+  if constexpr (R.r1 >= 0) cf *= in.c[R.r1];
+  if (mt.reversible[J]) {
+    double gr = in.G[R.r0];
+    if constexpr (R.r1 >= 0) gr *= in.G[R.r1];
+    if constexpr (dnu == 1) gr *= in.RTP;
+    if constexpr (dnu == -1) gr *= in.PRT;
+    double ap = in.iG[R.p0];
+    if constexpr (R.p1 >= 0) ap *= in.iG[R.p1];
+    cf = fma(-gr, ap, cf);
   }
+  double q = kf * cf;
   if constexpr (R.type == THIRD_BODY) q *= M;
   wdot[R.r0] -= q;
   if constexpr (R.r1 >= 0) wdot[R.r1] -= q;
@@ -210,19 +184,15 @@ __device__ __forceinline__ void reaction(const MechTables &mt, const RateInputs 
   if constexpr (R.p1 >= 0) wdot[R.p1] += q;
 }
 
-template <bool kDestr, int... J>
+template <int... J>
 __device__ __forceinline__ void all_reactions(const MechTables &mt, const RateInputs &in, double T,
-                                              double (&wdot)[NSP], double *dflux,
-                                              std::integer_sequence<int, J...>) {
-  (reaction<J, kDestr>(mt, in, T, wdot, dflux), ...);
+                                              double (&wdot)[NSP], std::integer_sequence<int, J...>) {
+  (reaction<J>(mt, in, T, wdot), ...);
 }
 
 // Molar production rates wdot (mol/m^3/s) at temperature T and clamped concentrations c.
-// kDestr: also the consumption fluxes per species into dflux (zeroed here).
-template <bool kDestr = false>
 __device__ __forceinline__ void production_rates(const MechTables &mt, double T,
-                                                 const double (&c)[NSP], double (&wdot)[NSP],
-                                                 double *dflux = nullptr) {
+                                                 const double (&c)[NSP], double (&wdot)[NSP]) {
   RateInputs in;
   in.lnT = log_t(T);
   in.invT = rcp2(T);
@@ -241,12 +211,11 @@ __device__ __forceinline__ void production_rates(const MechTables &mt, double T,
     // clamp keeps G finite far outside the tables' range
     g = clamp_abs(g, 700.0);
     in.G[k] = exp_t(-g);
-    in.iG[k] = kDestr ? rcp2(in.G[k]) : c[k] * rcp2(in.G[k]);
+    in.iG[k] = c[k] * rcp2(in.G[k]);
     wdot[k] = 0.0;
-    if constexpr (kDestr) dflux[k] = 0.0;
   }
   in.ctot = ctot;
-  all_reactions<kDestr>(mt, in, T, wdot, dflux, std::make_integer_sequence<int, NRX>{});
+  all_reactions(mt, in, T, wdot, std::make_integer_sequence<int, NRX>{});
 }
 
 // dY/dt of one cell at fixed (rho, e).  T: in = Newton guess, out = solved T.

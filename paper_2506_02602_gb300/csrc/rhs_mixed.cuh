@@ -170,46 +170,25 @@ struct RateInputsF {
   float c[NSP];
 };
 
-// fp32 transcendentals and divisions of the rate expressions: the CUDA library's
-// accurate functions for the integrator, or its fast intrinsics (hardware base-2
-// exponential and logarithm, approximate division; relative errors ~1e-6 on these
-// arguments) for the error test's estimator, which compares with a tolerance of ~5e-4 T.
-template <bool FAST>
-__device__ __forceinline__ float exp_r(float x) {
-  if constexpr (FAST) return __expf(x); else return expf(x);
-}
-template <bool FAST>
-__device__ __forceinline__ float log_r(float x) {
-  if constexpr (FAST) return __logf(x); else return logf(x);
-}
-template <bool FAST>
-__device__ __forceinline__ float log10_r(float x) {
-  if constexpr (FAST) return __log10f(x); else return log10f(x);
-}
-template <bool FAST>
-__device__ __forceinline__ float exp10_r(float x) {
-  if constexpr (FAST) return __exp10f(x); else return exp10f(x);
-}
-template <bool FAST>
-__device__ __forceinline__ float div_r(float a, float b) {
-  if constexpr (FAST) return __fdividef(a, b); else return a / b;
-}
-
-template <int J, bool FAST>
+// Troe broadening factor in fp32 on the fast intrinsics (hardware base-2 exponential and
+// logarithm, approximate division; relative errors ~1e-6 on these arguments), for the
+// estimators: the surrogate's error test, which compares with a tolerance of ~5e-4 T, and the
+// batched path's stiffness key.
+template <int J>
 __device__ __forceinline__ float troe_F_f32(const MechTables &mt, float T, float invT, float Pr) {
   constexpr int n = kRx[J].troe_n;
   if constexpr (n == 0) {
     return 1.0f;
   } else {
     const float a = mt.f.troe_a[J];
-    float Fc = (1.0f - a) * exp_r<FAST>(-T * mt.f.troe_i3[J]) + a * exp_r<FAST>(-T * mt.f.troe_i1[J]);
-    if constexpr (n == 4) Fc += exp_r<FAST>(-mt.f.troe_T2[J] * invT);
-    const float lFc = log10_r<FAST>(Fc);
+    float Fc = (1.0f - a) * __expf(-T * mt.f.troe_i3[J]) + a * __expf(-T * mt.f.troe_i1[J]);
+    if constexpr (n == 4) Fc += __expf(-mt.f.troe_T2[J] * invT);
+    const float lFc = __log10f(Fc);
     const float cc = -0.4f - 0.67f * lFc;
     const float nn = 0.75f - 1.27f * lFc;
-    const float x = log10_r<FAST>(Pr) + cc;
-    const float f1 = div_r<FAST>(x, nn - 0.14f * x);
-    return exp10_r<FAST>(div_r<FAST>(lFc, 1.0f + f1 * f1));
+    const float x = __log10f(Pr) + cc;
+    const float f1 = __fdividef(x, nn - 0.14f * x);
+    return __exp10f(__fdividef(lFc, 1.0f + f1 * f1));
   }
 }
 
@@ -317,12 +296,14 @@ __device__ __forceinline__ float ln_inv_kc(const GibbsF &g) {
   return q;
 }
 
-template <int J, bool FAST, typename Gibbs>
-__device__ __forceinline__ void reaction_mixed(const MechTables &mt, const RateInputsF &in,
-                                               const Gibbs &g, float (&wdot)[NSP]) {
+// One reaction in fp32 on the fast intrinsics, added into wdot.  With kDestr, the one-way
+// fluxes that consume each species are also summed into dflux (the stiffness key).
+template <int J, bool kDestr>
+__device__ __forceinline__ void reaction_f32(const MechTables &mt, const RateInputsF &in, const GibbsF &g,
+                                             float (&wdot)[NSP], float *dflux) {
   constexpr RxStruct R = kRx[J];
   float lnkf = fmaf(mt.f.beta[J], in.lnT, mt.f.lnA[J]) - mt.f.Ta[J] * in.invT;
-  float kf = mt.kconst[J] == 1 ? mt.f.A[J] : exp_r<FAST>(lnkf);
+  float kf = mt.kconst[J] == 1 ? mt.f.A[J] : __expf(lnkf);
   float M = 0.0f;
   if constexpr (R.type != ELEM) {
     M = in.ctot;
@@ -332,17 +313,17 @@ __device__ __forceinline__ void reaction_mixed(const MechTables &mt, const RateI
     }
   }
   if constexpr (R.type == FALLOFF) {
-    const float k0 = exp_r<FAST>(fmaf(mt.f.beta0[J], in.lnT, mt.f.lnA0[J]) - mt.f.Ta0[J] * in.invT);
-    const float Pr = div_r<FAST>(k0 * M, kf);
-    kf = (Pr > 0.0f) ? kf * div_r<FAST>(Pr, 1.0f + Pr) * troe_F_f32<J, FAST>(mt, in.T, in.invT, Pr) : 0.0f;
-    lnkf = log_r<FAST>(kf);
+    const float k0 = __expf(fmaf(mt.f.beta0[J], in.lnT, mt.f.lnA0[J]) - mt.f.Ta0[J] * in.invT);
+    const float Pr = __fdividef(k0 * M, kf);
+    kf = (Pr > 0.0f) ? kf * __fdividef(Pr, 1.0f + Pr) * troe_F_f32<J>(mt, in.T, in.invT, Pr) : 0.0f;
+    lnkf = __logf(kf);
   }
   float qf = kf * in.c[R.r0];
   if constexpr (R.r1 >= 0) qf *= in.c[R.r1];
-  float q = qf;
+  float q = qf, qr = 0.0f;
   if (mt.reversible[J]) {
-    const float kr = (kf > 0.0f) ? exp_r<FAST>(lnkf + ln_inv_kc<J>(g)) : 0.0f;
-    float qr = kr * in.c[R.p0];
+    const float kr = (kf > 0.0f) ? __expf(lnkf + ln_inv_kc<J>(g)) : 0.0f;
+    qr = kr * in.c[R.p0];
     if constexpr (R.p1 >= 0) qr *= in.c[R.p1];
     q = qf - qr;
   }
@@ -351,13 +332,20 @@ __device__ __forceinline__ void reaction_mixed(const MechTables &mt, const RateI
   if constexpr (R.r1 >= 0) wdot[R.r1] -= q;
   wdot[R.p0] += q;
   if constexpr (R.p1 >= 0) wdot[R.p1] += q;
+  if constexpr (kDestr) {
+    const float m = (R.type == THIRD_BODY) ? M : 1.0f;
+    dflux[R.r0] += m * qf;
+    if constexpr (R.r1 >= 0) dflux[R.r1] += m * qf;
+    dflux[R.p0] += m * qr;
+    if constexpr (R.p1 >= 0) dflux[R.p1] += m * qr;
+  }
 }
 
-template <bool FAST, typename Gibbs, int... J>
-__device__ __forceinline__ void all_reactions_mixed(const MechTables &mt, const RateInputsF &in,
-                                                    const Gibbs &g, float (&wdot)[NSP],
-                                                    std::integer_sequence<int, J...>) {
-  (reaction_mixed<J, FAST, Gibbs>(mt, in, g, wdot), ...);
+template <bool kDestr, int... J>
+__device__ __forceinline__ void all_reactions_f32(const MechTables &mt, const RateInputsF &in, const GibbsF &g,
+                                                  float (&wdot)[NSP], float *dflux,
+                                                  std::integer_sequence<int, J...>) {
+  (reaction_f32<J, kDestr>(mt, in, g, wdot, dflux), ...);
 }
 
 // What the rates need of the temperature, in fp64: T from the guess by solve_T, T, ln T and
@@ -702,10 +690,13 @@ __device__ __forceinline__ bool solve_T_f32(const MechTables &mt, const float (&
 }
 
 // dY/dt of one cell entirely in fp32 (temperature, Gibbs functions and ln(1/K_c)
-// included) with the fast intrinsics: the right-hand side of the surrogate's error test,
-// an estimator that needs relative accuracy far coarser than fp32's.  T: in = guess, out = solved T.
+// included) with the fast intrinsics: the right-hand side of the surrogate's error test and of
+// the stiffness key, estimators that need relative accuracy far coarser than fp32's.  T: in =
+// guess, out = solved T.  kDestr: also the consumption rates per unit concentration, D (0
+// where there is nothing to consume).
+template <bool kDestr = false>
 __device__ __forceinline__ bool cell_rhs_f32(const MechTables &mt, const float (&U)[NSP], float rho,
-                                             float invRho, float eR, float &T, float (&F)[NSP]) {
+                                             float invRho, float eR, float &T, float (&F)[NSP], float *D = nullptr) {
   float yw[NSP];
 #pragma unroll
   for (int k = 0; k < NSP; ++k) yw[k] = U[k] * mt.f.invW[k];
@@ -724,11 +715,15 @@ __device__ __forceinline__ bool cell_rhs_f32(const MechTables &mt, const float (
     in.c[k] = fmaxf(rho * yw[k], 0.0f);
     ctot += in.c[k];
     wdot[k] = 0.0f;
+    if constexpr (kDestr) D[k] = 0.0f;
   }
   in.ctot = ctot;
-  all_reactions_mixed<true>(mt, in, g, wdot, std::make_integer_sequence<int, NRX>{});
+  all_reactions_f32<kDestr>(mt, in, g, wdot, D, std::make_integer_sequence<int, NRX>{});
 #pragma unroll
-  for (int k = 0; k < NSP; ++k) F[k] = wdot[k] * mt.f.W[k] * invRho;
+  for (int k = 0; k < NSP; ++k) {
+    F[k] = wdot[k] * mt.f.W[k] * invRho;
+    if constexpr (kDestr) D[k] = in.c[k] > 1e-30f ? __fdividef(D[k], in.c[k]) : 0.0f;
+  }
   return true;
 }
 
