@@ -198,6 +198,30 @@ int build_tables(const chem_mechanism *m, MechTables *t) {
     t->has_eff[j] = any;
     t->eff_mask[j] = mask;
   }
+  // fixed-point forms of the rate coefficients
+  const double log2e = 1.4426950408889634;
+  t->fixed_ok = 1;
+  auto fixed = [&](double lnA, double b, double Ta, int64_t &qa, int64_t &qb, int64_t &qh) {
+    const double a2 = lnA * log2e, h2 = Ta * log2e;
+    if (!(std::fabs(a2) < 1000.0 && std::fabs(b) < 7.5 && std::fabs(h2) < 130000.0)) {
+      t->fixed_ok = 0;
+      return;
+    }
+    qa = (int64_t)std::ldexp(a2, 52);
+    qb = (int64_t)std::ldexp(b, 60);
+    qh = (int64_t)std::ldexp(h2, 46);
+  };
+  for (int j = 0; j < NRX; ++j) {
+    fixed(t->lnA[j], t->beta[j], t->Ta[j], t->qA[j], t->qB[j], t->qH[j]);
+    if (kRx[j].type != FALLOFF) continue;
+    fixed(t->lnA0[j], t->beta0[j], t->Ta0[j], t->qA0[j], t->qB0[j], t->qH0[j]);
+    t->troe_q3[j] = t->troe_i3[j] * log2e;
+    t->troe_q1[j] = t->troe_i1[j] * log2e;
+    t->troe_q2[j] = t->troe_T2[j] * log2e;
+  }
+  for (int r = 0; r < 2; ++r)
+    for (int k = 0; k < NSP; ++k)
+      for (int i = 0; i < 7; ++i) t->gc_q[r][k][i] = -log2e * t->gc[r][k][i];
   // element matrix (standard atomic masses of H, O, N)
   const double amass[CHEM_NUM_ELEMENTS] = {1.008e-3, 15.999e-3, 14.007e-3};
   for (int k = 0; k < NSP; ++k) {

@@ -131,6 +131,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_lsrk_persistent(const __grid_co
     load_mixed_tables<BLOCK>(mt);
     init_mixed_cols<BLOCK>(mixed_cols<BLOCK>());
   } else {
+    load_exp2_table();
     load_math_tables();
   }
   const unsigned FULL = 0xffffffffu;

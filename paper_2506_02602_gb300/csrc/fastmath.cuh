@@ -4,7 +4,8 @@
 //
 // On GB300 the FP64 pipe issues 2 lanes per clock per SM, and a library fp64 exp takes
 // about 20 of those slots (log about 37).  The right-hand side needs ~38 exponentials
-// and ~5 logarithms, so these two functions dominate its FP64 cost.  The versions here
+// and ~5 logarithms.  The exponentials run in fixed point on the integer pipe (exp2_q52); the
+// logarithms, and exponentials outside the fixed-point range,
 // follow Tang's table-driven methods (ACM TOMS 15 (1989) 144-157 for exp, 16 (1990)
 // 378-400 for log) with Taylor polynomials, in about 10 FP64 operations each; the
 // exponent and table-index arithmetic runs on the integer pipe and the 128-entry (exp)
@@ -44,9 +45,7 @@ __device__ __forceinline__ void load_math_tables() {
 // scale 2^m added to the exponent field of the table entry 2^(j/128) on the integer
 // pipe (10 FP64-pipe operations in all).  Arguments beyond +-710 are first clamped there
 // on the integer pipe, so they still give +inf above and a positive value below 1e-307
-// below, however large; a NaN stays NaN.  Kept out of line: the right-hand side calls it
-// ~38 times, and one shared copy keeps the kernel's code within the instruction cache
-// (measured 4 % faster than inlining it on GB300).
+// below, however large; a NaN stays NaN.  Kept out of line, one copy for its many calls.
 static __device__ __noinline__ double exp_t(double x) {
   const long long kLim = 0x40863000'00000000LL;  // 710.0
   const long long b = __double_as_longlong(x);
@@ -67,6 +66,77 @@ static __device__ __noinline__ double exp_t(double x) {
   const double tj = s_exp2_128[k & 127];
   const double ts = __hiloint2double(__double2hiint(tj) + ((k >> 7) << 20), __double2loint(tj));
   return fma(ts, p, ts);
+}
+
+// x clamped to [-lim, lim] for lim > 0 (a NaN gives +-lim)
+__device__ __forceinline__ double clamp_abs(double x, double lim) {
+  const long long b = __double_as_longlong(x);
+  const long long l = __double_as_longlong(lim);
+  return (b & 0x7fffffffffffffffLL) > l ? __longlong_as_double((b & (long long)0x8000000000000000ULL) | l) : x;
+}
+
+// ---- exponentials in fixed point, on the integer pipe ----
+// A 64-bit number in units of 2^-52 (Q52) stands for a base-2 logarithm: its 1/1024ths index
+// a table of 64-bit mantissas (8 KB in shared memory), and 2^r - 1 for the rest, r < 2^-10,
+// is u + u^2/2 in integer arithmetic with u = r ln2 (r in units of 2^-74) and the terms from
+// u^3 on in fp32.  No FP64 instruction: about 60 integer and wide-multiply instructions, 140
+// cycles of a sub-partition on GB300 against 640 for the table-driven exp_t, and at most
+// 0.6 ulp off.
+
+// Per-block copy of k_exp2_q63, filled by load_exp2_table().
+__shared__ unsigned long long s_exp2_q63[1024];
+
+__device__ __forceinline__ void load_exp2_table() {
+  for (int i = threadIdx.x; i < 1024; i += blockDim.x) s_exp2_q63[i] = k_exp2_q63[i];
+  __syncthreads();
+}
+
+__device__ __forceinline__ unsigned long long mul_wide(uint32_t a, uint32_t b) { return (unsigned long long)a * b; }
+
+// 2^(y 2^-52) for |y| < 1021 2^52.  Out of line, as exp_t: one copy of the code.
+static __device__ __noinline__ double exp2_q52(long long y) {
+  const uint32_t yl = (uint32_t)y;
+  const int yh = (int)(y >> 32), k = yh >> 10;
+  const uint32_t fh = __funnelshift_l(yl, (uint32_t)yh, 22), fl = yl << 22;  // r in units of 2^-74
+  const unsigned long long u = mul_wide(fh, kLn2Q64Hi) + __umulhi(fh, kLn2Q64Lo) + __umulhi(fl, kLn2Q64Hi);
+  const uint32_t uh = (uint32_t)(u >> 32), ul = (uint32_t)u;
+  const unsigned long long u2 = (mul_wide(uh, uh) >> 1) + __umulhi(uh, ul);  // u^2 / 2, units of 2^-84
+  const float g = (float)uh * 0x1p-42f;
+  const uint32_t c = (uint32_t)(g * g * g * fmaf(g, 0x1p64f / 24.0f, 0x1p64f / 6.0f));  // u^3/6 + u^4/24, 2^-64
+  const unsigned long long p = u + (u2 >> 10) + ((unsigned long long)c << 10);          // 2^r - 1, 2^-74
+  const unsigned long long t = s_exp2_q63[k & 1023];
+  const uint32_t th = (uint32_t)(t >> 32), tl = (uint32_t)t, ph = (uint32_t)(p >> 32), pl = (uint32_t)p;
+  const unsigned long long tp = mul_wide(th, ph) + __umulhi(th, pl) + __umulhi(tl, ph);  // 2^-73
+  const unsigned long long m = (t + (tp >> 10) + 0x400ull) >> 11;  // 53 bits, rounded; carries into the exponent
+  return __longlong_as_double((long long)((unsigned long long)(uint32_t)((k >> 10) + 1022) << 52) + (long long)m);
+}
+
+// |x| in units of 2^-Q, truncated, for |x| < 2^(62 - Q + 1).
+template <int Q>
+__device__ __forceinline__ unsigned long long abs_q(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ff) - 1023;
+  const unsigned long long m = ((b & 0x000fffffffffffffull) | 0x0010000000000000ull) << 10;
+  return m >> min(62 - Q - e, 63);
+}
+
+// x in Q52, limited to +-1009.9 (a factor e^+-700)
+__device__ __forceinline__ long long to_q52(double x) {
+  const long long v = (long long)abs_q<52>(clamp_abs(x, 1009.875));
+  return __double2hiint(x) < 0 ? -v : v;
+}
+
+// 2^x, |x| limited as above
+__device__ __forceinline__ double exp2_lim(double x) { return exp2_q52(to_q52(x)); }
+
+// Arrhenius: A T^b exp(-Ta / T) from log2 A (Q52), b (Q60), Ta / ln2 (Q46), log2 T (Q58) and
+// 1 / T (Q70) for T in (128, 32768): the exponent is exact to 2^-51.
+__device__ __forceinline__ long long arrhenius_log2(long long a, long long b, long long h, long long lT, long long iT) {
+  return a + (__mul64hi(b, lT) >> 2) - __mul64hi(h, iT);
+}
+__device__ __forceinline__ long long limit_q52(long long y) {
+  const long long lim = 1019ll << 52;
+  return min(max(y, -lim), lim);
 }
 
 // log(x) for positive normal finite x.
@@ -175,13 +245,6 @@ __device__ __forceinline__ double max_abs(double a, double b) {
 __device__ __forceinline__ double clamp_nonneg(double x) {
   const long long b = __double_as_longlong(x);
   return __longlong_as_double(b & ~(b >> 63));
-}
-
-// x clamped to [-lim, lim] for lim > 0 (a NaN gives +-lim)
-__device__ __forceinline__ double clamp_abs(double x, double lim) {
-  const long long b = __double_as_longlong(x);
-  const long long l = __double_as_longlong(lim);
-  return (b & 0x7fffffffffffffffLL) > l ? __longlong_as_double((b & (long long)0x8000000000000000ULL) | l) : x;
 }
 
 // x = hi + lo for an fp64 x of magnitude below 2^12: hi is x truncated to a multiple of

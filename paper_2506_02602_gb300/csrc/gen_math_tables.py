@@ -4,6 +4,8 @@ exp (Tang 1989, "Table-driven implementation of the exponential function in IEEE
 floating-point arithmetic"): x = (128 m + j) ln2/128 + r, exp(x) = 2^m 2^(j/128) e^r with
 |r| <= ln2/256; the table holds 2^(j/128), j = 0..127, each correctly rounded.
 
+exp2 in fixed point (exp2_q52): 2^(j/1024), j = 0..1023, rounded to 64-bit integers in units of 2^-63.
+
 log (Tang 1990, "Table-driven implementation of the logarithm function"): x = 2^e f,
 f in [1, 2), c_j = RN(1 / (1 + j/64)) with j the nearest 64th of f - 1, r = f c_j - 1
 (one FMA), log x = e ln2 + L_j + log1p(r) with L_j = -ln(c_j) correctly rounded for the
@@ -45,6 +47,12 @@ def main():
     for j in range(128):
         out.append(f"    {hexd((Decimal(j) / 128 * LN2).exp())},")
     out.append("};")
+    out.append("// 2^(j/1024) in units of 2^-63, j = 0..1023")
+    out.append("__device__ const unsigned long long k_exp2_q63[1024] = {")
+    for j in range(1024):
+        v = int(((Decimal(j) / 1024 * LN2).exp() * 2**63).to_integral_value())
+        out.append(f"    {v:#018x}ull,")
+    out.append("};")
     inv = [float(1 / (1 + Decimal(j) / 64)) for j in range(65)]
     out.append("// c_j = RN(1 / (1 + j/64)), j = 0..64")
     out.append("__device__ const double k_log_inv[65] = {")
@@ -77,6 +85,8 @@ def main():
         f"constexpr double kInvLn2x128 = {hexd(128 / LN2)};",
         f"constexpr double kLn2d128Hi = {float(LN2 / 128).hex()};",
         f"constexpr double kLn2d128Lo = {hexd(LN2 / 128 - Decimal(float(LN2 / 128)))};",
+        f"constexpr double kLog2E = {hexd(1 / LN2)}, kLog2_10 = {hexd(Decimal(10).ln() / LN2)};",
+        f"constexpr unsigned kLn2Q64Hi = {int(LN2 * 2**64) >> 32:#x}u, kLn2Q64Lo = {int(LN2 * 2**64) & 0xffffffff:#x}u;",
         f"constexpr float kLn2A = {ln2a.hex()}f, kLn2B = {ln2b.hex()}f, kLn2C = {ln2c.hex()}f;",
         f"constexpr double kLn10 = {hexd(Decimal(10).ln())};",
         f"constexpr double kInvLn10 = {hexd(1 / Decimal(10).ln())};",

@@ -20,6 +20,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_lsrk(const __grid_constant__ Me
     load_mixed_tables<BLOCK>(mt);
     init_mixed_cols<BLOCK>(mixed_cols<BLOCK>());
   } else {
+    load_exp2_table();
     load_math_tables();
   }
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

@@ -87,6 +87,13 @@ struct MechTables {
   // fall-off low-pressure limit and Troe parameters (alpha, 1/T***, 1/T*, T**)
   double lnA0[NRX], beta0[NRX], Ta0[NRX];
   double troe_a[NRX], troe_i3[NRX], troe_i1[NRX], troe_T2[NRX];
+  // the same for the fixed-point exponentials (fastmath.cuh): log2 A (Q52), b (Q60),
+  // Ta / ln2 (Q46) of both limits, the Gibbs polynomials times -log2(e) and the Troe
+  // temperatures' factors times log2(e); fixed_ok: every coefficient is in their range
+  int64_t qA[NRX], qB[NRX], qH[NRX], qA0[NRX], qB0[NRX], qH0[NRX];
+  double gc_q[2][NSP][7];
+  double troe_q3[NRX], troe_q1[NRX], troe_q2[NRX];
+  int32_t fixed_ok;
   // third-body efficiencies minus one: [M] = sum_k c_k + sum_k effm1 c_k
   double effm1[NRX][NSP];
   int32_t has_eff[NRX];
