@@ -65,14 +65,16 @@ typedef enum {
 } chem_cell_status;
 
 typedef enum {
-  CHEM_VARIANT_FP64 = 0,  /* every value in fp64 (reciprocals by Newton-Raphson refinement
-                             of the hardware approximation, within 2 ulp except in the
-                             temperature solve's step, 2^-40; that solve's stop test
-                             compares the fp32-rounded step and temperature) */
-  CHEM_VARIANT_MIXED = 1  /* rates and RK stage derivatives in fp32; temperature solve,
-                             Gibbs functions, solution and error registers and step
-                             control in fp64; ln(1/K_c) is the fp64 sum of the Gibbs
-                             terms rounded once to fp32 for the fp32 reverse rate */
+  CHEM_VARIANT_FP64 = 0,  /* every value in fp64 or in 64-bit fixed point with no larger an
+                             error (sums of products, exponentials, logarithms; reciprocals
+                             by Newton-Raphson refinement of the hardware approximation,
+                             within 2 ulp; the temperature solve's steps have an fp32 slope
+                             and end at 4e-9 T, the root exact to ~2e-15) */
+  CHEM_VARIANT_MIXED = 1  /* rates and RK stage derivatives in fp32; solution and error
+                             registers and step control in fp64; temperature solve and Gibbs
+                             functions in double-float, redone in fp64 where the fp32 rounding
+                             of T, ln T, 1/T or ln(1/K_c) is in doubt; ln(1/K_c) is rounded
+                             once to fp32 for the fp32 reverse rate */
 } chem_variant;
 
 /*
@@ -657,8 +659,8 @@ int chem_diag_fma_peak(int op, int32_t blocks, int32_t threads, int64_t iters, v
  * (device, n * n_reactions fp64, row i = temperature i, the fp32 results widened
  * exactly), as the mixed-precision right-hand sides form them: form 0 the mixed
  * variant's (fp64 Gibbs functions summed as fp32 hi/lo pairs), form 1 the all-fp32 one of
- * the surrogate's error test.  The plain fp64 variant never forms ln K_c (it multiplies
- * exp(-g_k / (R_u T)) factors) and has no form here.  Errors: NULL ctx, form not 0 or 1,
+ * the surrogate's error test.  The plain fp64 variant forms log2 K_c in fixed point and
+ * has no form here.  Errors: NULL ctx, form not 0 or 1,
  * n outside [0, 2^30] or NULL pointers with n > 0 -> CHEM_ERR_INVALID; a failed launch ->
  * CHEM_ERR_CUDA.  Asynchronous on stream.
  */

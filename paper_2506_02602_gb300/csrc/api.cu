@@ -198,18 +198,23 @@ int build_tables(const chem_mechanism *m, MechTables *t) {
     t->has_eff[j] = any;
     t->eff_mask[j] = mask;
   }
-  // fixed-point forms of the rate coefficients
+  // fixed-point forms: every sum of products below stays inside 64 bits for T in (128, 8192) K,
+  // |Y| < 1.25 and rho in (2^-64, 2^64) when the magnitudes here are below their bounds
   const double log2e = 1.4426950408889634;
-  t->fixed_ok = 1;
-  auto fixed = [&](double lnA, double b, double Ta, int64_t &qa, int64_t &qb, int64_t &qh) {
+  t->fixed_ok = Tmid > 128.0 && Tmid < 8192.0;
+  auto qcoef = [](double v, int q, int drop) {
+    const int64_t x = (int64_t)std::ldexp(v, q);
+    return QCoef{(int32_t)(x >> 32), (int32_t)((uint32_t)x >> drop)};
+  };
+  auto fixed = [&](double lnA, double b, double Ta, int64_t &qa, QCoef &qb, QCoef &qh) {
     const double a2 = lnA * log2e, h2 = Ta * log2e;
-    if (!(std::fabs(a2) < 1000.0 && std::fabs(b) < 7.5 && std::fabs(h2) < 130000.0)) {
+    if (!(std::fabs(a2) < 700.0 && std::fabs(b) < 7.5 && std::fabs(h2) < 130000.0)) {
       t->fixed_ok = 0;
       return;
     }
     qa = (int64_t)std::ldexp(a2, 52);
-    qb = (int64_t)std::ldexp(b, 60);
-    qh = (int64_t)std::ldexp(h2, 46);
+    qb = qcoef(b, 58, 2);
+    qh = qcoef(-h2, 46, 2);
   };
   for (int j = 0; j < NRX; ++j) {
     fixed(t->lnA[j], t->beta[j], t->Ta[j], t->qA[j], t->qB[j], t->qH[j]);
@@ -219,9 +224,40 @@ int build_tables(const chem_mechanism *m, MechTables *t) {
     t->troe_q1[j] = t->troe_i1[j] * log2e;
     t->troe_q2[j] = t->troe_T2[j] * log2e;
   }
-  for (int r = 0; r < 2; ++r)
-    for (int k = 0; k < NSP; ++k)
-      for (int i = 0; i < 7; ++i) t->gc_q[r][k][i] = -log2e * t->gc[r][k][i];
+  for (int r = 0; r < 2 && t->fixed_ok; ++r) {
+    int S = 13;
+    if (r == 0) while (std::ldexp(1.0, S - 1) >= Tmid) --S;
+    t->q_log2[r] = S;
+    double esum = 0.0, ei[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int k = 0; k < NSP; ++k) {
+      for (int i = 0; i < 6; ++i) {
+        const double v = i < 5 ? std::ldexp(t->ecw[r][k][i], S * (i + 1)) : t->ecw[r][k][5];
+        ei[i] += std::fabs(v);
+        esum += std::fabs(v);
+        if (std::fabs(v) < 0x1p26) t->qe[r][k][i] = qcoef(v, 37, 2);
+        else t->fixed_ok = 0;
+      }
+      const double *g = t->gc[r][k];
+      double gsum = 13.0 * std::fabs(g[0]) + std::fabs(g[5]) * log2e / 128.0 + std::fabs(g[0] + g[6]) * log2e;
+      double gt[4];
+      for (int i = 0; i < 4; ++i) {
+        gt[i] = std::ldexp(-log2e * g[i + 1], S * (i + 1));
+        gsum += std::fabs(gt[i]);
+        if (!(std::fabs(gt[i]) < 64.0)) t->fixed_ok = 0;
+      }
+      if (!(gsum < 1500.0) || !(std::fabs(g[0]) < 64.0)) t->fixed_ok = 0;
+      if (!t->fixed_ok) break;
+      t->qg[r][k][0] = qcoef(g[0], 56, 2);
+      t->qg[r][k][1] = qcoef(-log2e * g[5], 44, 2);
+      for (int i = 0; i < 4; ++i) t->qgt[r][k][i] = qcoef(gt[i], 57, 4);
+      t->qg1[r][k] = (int64_t)std::ldexp(-log2e * (g[0] + g[6]), 50);
+    }
+    for (int i = 0; i < 6; ++i)
+      if (!(ei[i] < 0x1p26 * 1.4)) t->fixed_ok = 0;
+    if (!(esum < 0x1.4p28 * 1.1)) t->fixed_ok = 0;
+  }
+  if (t->fixed_ok) t->qT_mid = (int64_t)std::ldexp(Tmid, 50);
+  t->qRP = (int64_t)std::ldexp(std::log2(R_U / P_REF), 50);
   // element matrix (standard atomic masses of H, O, N)
   const double amass[CHEM_NUM_ELEMENTS] = {1.008e-3, 15.999e-3, 14.007e-3};
   for (int k = 0; k < NSP; ++k) {

@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_lsrk_persistent(const __grid_co
     load_mixed_tables<BLOCK>(mt);
     init_mixed_cols<BLOCK>(mixed_cols<BLOCK>());
   } else {
-    load_exp2_table();
+    load_fixed_tables(mt);
     load_math_tables();
   }
   const unsigned FULL = 0xffffffffu;
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_lsrk_persistent(const __grid_co
           c.t = 0.0;  // next substep from the current state; h and the T guess carry
           c.done = false;
         } else {
-          cell_finish(mt, c);
+          cell_finish<V, BLOCK>(mt, c);
 #pragma unroll
           for (int k = 0; k < NSP; ++k) a.Y[k * a.ld + cell] = c.X[k];
           a.T[cell] = c.T;
@@ -234,10 +234,8 @@ static const void *persistent_kernel(int variant, int shape) {
                                        : persistent_fn<CHEM_VARIANT_FP64>(shape);
 }
 
-// Dynamic shared memory of a shape: the mixed variant's per-thread columns.
-static size_t persistent_smem(int variant, int shape) {
-  return variant == CHEM_VARIANT_MIXED ? mixed_cols_bytes(kShapeBlock[shape]) : 0;
-}
+// Dynamic shared memory of a shape: the variant's per-thread columns.
+static size_t persistent_smem(int variant, int shape) { return cols_bytes(variant, kShapeBlock[shape]); }
 
 // Resident CTAs per SM and registers per thread of every (variant, shape), per device
 // ordinal (looked up once; 0 = not yet).

@@ -3,12 +3,13 @@
 // persistent work-stealing kernel (one attempt per iteration, lanes refilled as cells
 // finish) run the same arithmetic.
 //
-// Per cell the integrator keeps four register vectors of NSP values: the solution
+// Per cell the integrator keeps four vectors of NSP values: the solution
 // register X (y_n advancing to y_n+1), the stage register U (input of the next
 // right-hand side), the error register E (sum_i (b_i - bhat_i) h F_i, the embedded
 // third-order estimate) and the saved y_n for a rejected step; F is transient.  That is
 // the two-register scheme of Eq. 21 plus the error register the paper adds, plus the
-// copy any rejecting controller needs.  The stage loop stays rolled (coefficients from
+// copy any rejecting controller needs.  X, U and E are per-thread columns of shared memory
+// (a stage touches each value a few times; in registers they crowd the right-hand side).  The stage loop stays rolled (coefficients from
 // __constant__), so the right-hand side is inlined once.
 //
 // Controller (Eq. 22): ||e|| = sqrt(mean_k (E_k / (rtol max(|y_n,k|, |y_n+1,k|) + atol))^2);
@@ -17,7 +18,7 @@
 // 1e-15 dt is an underflow.  A trial stage whose temperature solve fails rejects the
 // attempt with factor 1/5; a failure at stage 1 (the accepted state) ends the cell.
 //
-// Variants: V = CHEM_VARIANT_FP64, every register fp64; V = CHEM_VARIANT_MIXED
+// Variants: V = CHEM_VARIANT_FP64, every vector fp64; V = CHEM_VARIANT_MIXED
 // (cell_attempt_mixed), the stage register U and the stage derivative F are fp32
 // (cell_rhs_mixed) while X, y_n, E, the WRMS norm and the controller stay fp64.
 #pragma once
@@ -150,37 +151,40 @@ __device__ __forceinline__ bool attempt_end(CellState &c, double h, double sum) 
 }
 
 // One attempted step (or the end of the integration), fp64 variant.  Sets c.done when the
-// cell has reached dt or hit a limit.
+// cell has reached dt or hit a limit.  c.X holds the saved y_n, in local memory (the loops that
+// index it are rolled): four accesses a species and step.
+template <int ST>
 __device__ __forceinline__ void cell_attempt_fp64(const MechTables &mt, CellState &c,
                                                   const StepParams &p) {
   double h;
   if (!attempt_begin(c, p, h)) return;
-  double Xs[NSP], E[NSP], U[NSP];
-#pragma unroll
+  const Fp64Cols m = fp64_cols<ST>();
+#pragma unroll 1
   for (int k = 0; k < NSP; ++k) {
-    Xs[k] = c.X[k];
-    U[k] = c.X[k];
-    E[k] = 0.0;
+    const double x = c.X[k];
+    m.X[k * ST] = x;
+    m.U[k * ST] = x;
+    m.E[k * ST] = 0.0;
   }
   int failed = 0;
-  double Tacc = c.T;  // temperature of the accepted state, set by stage 1
+  double T = c.T, Tacc = T;  // temperature of the accepted state, set by stage 1
 #pragma unroll 1
   for (int s = 0; s < 5; ++s) {
     double F[NSP];
     ++c.nrhs;
-    if (!cell_rhs(mt, U, c.rho, c.invRho, c.eR, c.T, F)) { failed = s + 1; break; }
-    if (s == 0) Tacc = c.T;
+    if (!cell_rhs<ST>(mt, m, c.rho, c.invRho, c.eR, T, F)) { failed = s + 1; break; }
+    if (s == 0) Tacc = T;
     const double ha = h * c_ls_a[s], hb = h * c_ls_b[s], he = h * c_ls_e[s];
 #pragma unroll
     for (int k = 0; k < NSP; ++k) {
-      E[k] = fma(he, F[k], E[k]);
-      U[k] = fma(ha, F[k], c.X[k]);
-      c.X[k] = fma(hb, F[k], c.X[k]);
+      const double x = m.X[k * ST];
+      m.E[k * ST] = fma(he, F[k], m.E[k * ST]);
+      m.U[k * ST] = fma(ha, F[k], x);
+      m.X[k * ST] = fma(hb, F[k], x);
     }
   }
   if (failed == 1) {
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) c.X[k] = Xs[k];
+    c.T = T;
     c.status = CHEM_CELL_NEWTON_FAIL;
     c.done = true;
     return;
@@ -189,18 +193,20 @@ __device__ __forceinline__ void cell_attempt_fp64(const MechTables &mt, CellStat
   double sum = CUDART_NAN;
   if (!failed) {
     sum = 0.0;
-#pragma unroll
+#pragma unroll kRoll
     for (int k = 0; k < NSP; ++k) {
-      const double w = E[k] * rcp2(fma(p.rtol, max_abs(Xs[k], c.X[k]), p.atol));
+      const double w = m.E[k * ST] * rcp2(fma(p.rtol, max_abs(c.X[k], m.X[k * ST]), p.atol));
       sum = fma(w, w, sum);
     }
   }
   // a rejected attempt returns the cell to its accepted state, the temperature warm
   // start included (a trial stage's temperature can sit near another root of e(T) of the
   // extrapolated polynomials)
-  if (!attempt_end(c, h, sum)) {
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) c.X[k] = Xs[k];
+  if (attempt_end(c, h, sum)) {
+#pragma unroll 1
+    for (int k = 0; k < NSP; ++k) c.X[k] = m.X[k * ST];
+    c.T = T;
+  } else {
     c.T = Tacc;
   }
 }
@@ -268,10 +274,15 @@ __device__ __forceinline__ void cell_attempt_mixed(const MechTables &mt, CellSta
   }
 }
 
+// Dynamic shared memory of a block: the variant's columns.
+constexpr size_t cols_bytes(int variant, int block) {
+  return variant == CHEM_VARIANT_MIXED ? mixed_cols_bytes(block) : fp64_cols_bytes(block);
+}
+
 template <int V, int BLOCK>
 __device__ __forceinline__ void cell_attempt(const MechTables &mt, CellState &c, const StepParams &p) {
   if constexpr (V == CHEM_VARIANT_MIXED) cell_attempt_mixed<BLOCK>(mt, c, p);
-  else cell_attempt_fp64(mt, c, p);
+  else cell_attempt_fp64<BLOCK>(mt, c, p);
 }
 
 // One attempted step of a full-storage scheme (CHEM_SCHEME_FULL_STORAGE: table 0, five
@@ -335,7 +346,10 @@ __device__ __forceinline__ void cell_attempt_full(const MechTables &mt, CellStat
       for (int k = 0; k < NSP; ++k) F[k] = m.Q[k * BLOCK];
       c.T = ff2d(Tf);
     } else {
-      ok = cell_rhs(mt, U, c.rho, c.invRho, c.eR, c.T, F);
+      const Fp64Cols m = fp64_cols<BLOCK>();
+#pragma unroll
+      for (int k = 0; k < NSP; ++k) m.U[k * BLOCK] = U[k];
+      ok = cell_rhs<BLOCK>(mt, m, c.rho, c.invRho, c.eR, c.T, F);
     }
     if (!ok) { failed = s + 1; break; }
     if (s == 0) Tacc = c.T;
@@ -394,9 +408,17 @@ __device__ __forceinline__ void cell_attempt_full(const MechTables &mt, CellStat
   c.h = h * fac;
 }
 
-// Temperature of the final state (fp64 Newton); a failure marks the cell.
+// Temperature of the final state; a failure marks the cell.  The mixed variant keeps the fp64
+// Newton.
+template <int V, int BLOCK>
 __device__ __forceinline__ void cell_finish(const MechTables &mt, CellState &c) {
   if (c.status == CHEM_CELL_NONFINITE) return;
+  if constexpr (V == CHEM_VARIANT_FP64) {
+    const Fp64Cols m = fp64_cols<BLOCK>();
+#pragma unroll
+    for (int k = 0; k < NSP; ++k) m.U[k * BLOCK] = c.X[k];
+    if (mt.fixed_ok && solve_T_fixed<BLOCK>(mt, m.U, c.eR, c.T)) return;
+  }
   if (!solve_T(mt, c.X, c.eR, c.T)) {
     if (c.status == CHEM_CELL_OK) c.status = CHEM_CELL_NEWTON_FAIL;
     c.T = CUDART_NAN;

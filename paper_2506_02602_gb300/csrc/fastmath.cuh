@@ -3,9 +3,9 @@
 // clamps on the integer pipe.
 //
 // On GB300 the FP64 pipe issues 2 lanes per clock per SM, and a library fp64 exp takes
-// about 20 of those slots (log about 37).  The right-hand side needs ~38 exponentials
-// and ~5 logarithms.  The exponentials run in fixed point on the integer pipe (exp2_q52); the
-// logarithms, and exponentials outside the fixed-point range,
+// about 20 of those slots (log about 37).  The right-hand side's ~50 exponentials, its logarithms
+// and its sums of products run in 64-bit fixed point on the integer pipe (exp2_q52, log2_q58,
+// DotQ).  Arguments outside the fixed-point forms' ranges take exp_t and log_t, which
 // follow Tang's table-driven methods (ACM TOMS 15 (1989) 144-157 for exp, 16 (1990)
 // 378-400 for log) with Taylor polynomials, in about 10 FP64 operations each; the
 // exponent and table-index arithmetic runs on the integer pipe and the 128-entry (exp)
@@ -93,8 +93,8 @@ __device__ __forceinline__ void load_exp2_table() {
 
 __device__ __forceinline__ unsigned long long mul_wide(uint32_t a, uint32_t b) { return (unsigned long long)a * b; }
 
-// 2^(y 2^-52) for |y| < 1021 2^52.  Out of line, as exp_t: one copy of the code.
-static __device__ __noinline__ double exp2_q52(long long y) {
+// 2^(y 2^-52) for |y| < 1021 2^52
+__device__ __forceinline__ double exp2_q52_body(long long y) {
   const uint32_t yl = (uint32_t)y;
   const int yh = (int)(y >> 32), k = yh >> 10;
   const uint32_t fh = __funnelshift_l(yl, (uint32_t)yh, 22), fl = yl << 22;  // r in units of 2^-74
@@ -109,6 +109,13 @@ static __device__ __noinline__ double exp2_q52(long long y) {
   const unsigned long long tp = mul_wide(th, ph) + __umulhi(th, pl) + __umulhi(tl, ph);  // 2^-73
   const unsigned long long m = (t + (tp >> 10) + 0x400ull) >> 11;  // 53 bits, rounded; carries into the exponent
   return __longlong_as_double((long long)((unsigned long long)(uint32_t)((k >> 10) + 1022) << 52) + (long long)m);
+}
+
+// Out of line, as exp_t: one copy of the code; two at a time where there are two, whose chains
+// of dependent instructions then overlap.
+static __device__ __noinline__ double exp2_q52(long long y) { return exp2_q52_body(y); }
+static __device__ __noinline__ double2 exp2_q52(long long y0, long long y1) {
+  return make_double2(exp2_q52_body(y0), exp2_q52_body(y1));
 }
 
 // |x| in units of 2^-Q, truncated, for |x| < 2^(62 - Q + 1).
@@ -126,14 +133,70 @@ __device__ __forceinline__ long long to_q52(double x) {
   return __double2hiint(x) < 0 ? -v : v;
 }
 
-// 2^x, |x| limited as above
-__device__ __forceinline__ double exp2_lim(double x) { return exp2_q52(to_q52(x)); }
+// ---- sums of products in fixed point ----
+// A 64-bit number is split into its upper 32 bits (signed) and the top 32 - D of its lower 32
+// bits; of the product of two such numbers the upper x upper part and the two cross parts
+// accumulate in 64 bits, one IMAD.WIDE each and nothing else: 15 cycles of a sub-partition a
+// term on GB300 against 64 for an FP64 multiply-add.  What is dropped is below 2^(2 D - 64) of
+// a unit of the result; callers bound their operands so that neither sum overflows.
+template <int D>
+struct Limbs { int h, l; };
 
-// Arrhenius: A T^b exp(-Ta / T) from log2 A (Q52), b (Q60), Ta / ln2 (Q46), log2 T (Q58) and
-// 1 / T (Q70) for T in (128, 32768): the exponent is exact to 2^-51.
-__device__ __forceinline__ long long arrhenius_log2(long long a, long long b, long long h, long long lT, long long iT) {
-  return a + (__mul64hi(b, lT) >> 2) - __mul64hi(h, iT);
+template <int D>
+__device__ __forceinline__ Limbs<D> limbs(long long v) { return {(int)(v >> 32), (int)((uint32_t)v >> D)}; }
+
+template <int D>
+struct DotQ {
+  long long h, x;
+  __device__ __forceinline__ void add(int ch, int cl, const Limbs<D> &p) {
+    h += (long long)ch * p.h;
+    x += (long long)ch * p.l;
+    x += (long long)cl * p.h;
+  }
+  __device__ __forceinline__ long long value() const { return h + (x >> (32 - D)); }  // sum / 2^64
+};
+
+// m t 2^-63 for 0 <= t < 2^63
+__device__ __forceinline__ long long mul_q63(long long m, long long t) {
+  const int mh = (int)(m >> 32), ml = (int)((uint32_t)m >> 1), th = (int)(t >> 32), tl = (int)((uint32_t)t >> 1);
+  return (((long long)mh * th) << 1) + (((long long)mh * tl + (long long)ml * th) >> 30);
 }
+
+// Per-block copies of k_log2_c and k_log2_q58, filled by load_log2_table().
+__shared__ unsigned short s_log2_c[256];
+__shared__ long long s_log2_q58[256];
+
+__device__ __forceinline__ void load_log2_table() {
+  for (int i = threadIdx.x; i < 256; i += blockDim.x) {
+    s_log2_c[i] = k_log2_c[i];
+    s_log2_q58[i] = k_log2_q58[i];
+  }
+  __syncthreads();
+}
+
+// log2 x in units of 2^-58 for positive normal x, at most 8 units off: x = 2^e f, r = f c_j - 1
+// exact in units of 2^-67 (|r| < 2^-8.9), log2(1 + r) with the terms from r^4 on in fp32.
+static __device__ __noinline__ long long log2_q58(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)(b >> 52) - 1023, j = (int)(b >> 44) & 255;
+  const unsigned long long f = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
+  const long long r = (long long)((f * s_log2_c[j]) << 4);  // units of 2^-71; the 1 drops out
+  const long long u = __mul64hi(r, kLog2E_q62);               // r log2(e), 2^-69
+  const long long r2 = __mul64hi(r, r);                       // r^2, 2^-78
+  const long long t = __mul64hi(r2, kLog2E_q62);              // r^2 log2(e) / 2, 2^-77
+  const long long c = __mul64hi(__mul64hi(r2, r), kLog2EThird_q64);  // r^3 log2(e) / 3, 2^-85
+  const float rf = (float)(int)(r >> 32) * 0x1p-39f, rf2 = rf * rf;
+  const float d = rf2 * rf2 * (0x1p58f * (float)kLog2E) * fmaf(rf, 0.2f, -0.25f);
+  return ((long long)e << 58) + s_log2_q58[j] + (u >> 11) - (t >> 19) + (c >> 27) + (long long)(int)d;
+}
+
+// x 2^-50 for x in (2^57, 2^63)
+__device__ __forceinline__ double q50_to_double(long long x) {
+  const int n = __clz((int)(x >> 32));  // 1..6
+  const unsigned long long m = ((unsigned long long)x + (1ull << (10 - n))) >> (11 - n);
+  return __longlong_as_double(((long long)(1035 - n) << 52) + (long long)m);  // the leading one adds to the exponent
+}
+
 __device__ __forceinline__ long long limit_q52(long long y) {
   const long long lim = 1019ll << 52;
   return min(max(y, -lim), lim);

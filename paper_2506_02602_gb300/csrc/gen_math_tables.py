@@ -6,6 +6,9 @@ floating-point arithmetic"): x = (128 m + j) ln2/128 + r, exp(x) = 2^m 2^(j/128)
 
 exp2 in fixed point (exp2_q52): 2^(j/1024), j = 0..1023, rounded to 64-bit integers in units of 2^-63.
 
+log2 in fixed point (log2_q58): c_j = 2^15 / (1 + (j + 1/2) / 256), j = 0..255, rounded to
+integers, and -log2(c_j 2^-15) of the rounded c_j in units of 2^-58.
+
 log (Tang 1990, "Table-driven implementation of the logarithm function"): x = 2^e f,
 f in [1, 2), c_j = RN(1 / (1 + j/64)) with j the nearest 64th of f - 1, r = f c_j - 1
 (one FMA), log x = e ln2 + L_j + log1p(r) with L_j = -ln(c_j) correctly rounded for the
@@ -53,6 +56,18 @@ def main():
         v = int(((Decimal(j) / 1024 * LN2).exp() * 2**63).to_integral_value())
         out.append(f"    {v:#018x}ull,")
     out.append("};")
+    cq = [int((2**15 / (1 + (j + Decimal(1) / 2) / 256)).to_integral_value()) for j in range(256)]
+    out.append("// c_j = RN(2^15 / (1 + (j + 1/2) / 256)), j = 0..255")
+    out.append("__device__ const unsigned short k_log2_c[256] = {")
+    for j in range(0, 256, 8):
+        out.append("    " + " ".join(f"{c}," for c in cq[j:j + 8]))
+    out.append("};")
+    out.append("// -log2(c_j 2^-15) in units of 2^-58")
+    out.append("__device__ const long long k_log2_q58[256] = {")
+    for c in cq:
+        v = int((-(Decimal(c) / 2**15).ln() / LN2 * 2**58).to_integral_value())
+        out.append(f"    {v}ll,")
+    out.append("};")
     inv = [float(1 / (1 + Decimal(j) / 64)) for j in range(65)]
     out.append("// c_j = RN(1 / (1 + j/64)), j = 0..64")
     out.append("__device__ const double k_log_inv[65] = {")
@@ -87,6 +102,8 @@ def main():
         f"constexpr double kLn2d128Lo = {hexd(LN2 / 128 - Decimal(float(LN2 / 128)))};",
         f"constexpr double kLog2E = {hexd(1 / LN2)}, kLog2_10 = {hexd(Decimal(10).ln() / LN2)};",
         f"constexpr unsigned kLn2Q64Hi = {int(LN2 * 2**64) >> 32:#x}u, kLn2Q64Lo = {int(LN2 * 2**64) & 0xffffffff:#x}u;",
+        f"constexpr long long kLog2E_q62 = {int((1 / LN2 * 2**62).to_integral_value()):#x}ll;",
+        f"constexpr long long kLog2EThird_q64 = {int((1 / LN2 / 3 * 2**64).to_integral_value()):#x}ll;",
         f"constexpr float kLn2A = {ln2a.hex()}f, kLn2B = {ln2b.hex()}f, kLn2C = {ln2c.hex()}f;",
         f"constexpr double kLn10 = {hexd(Decimal(10).ln())};",
         f"constexpr double kInvLn10 = {hexd(1 / Decimal(10).ln())};",

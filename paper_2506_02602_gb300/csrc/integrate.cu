@@ -20,7 +20,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_lsrk(const __grid_constant__ Me
     load_mixed_tables<BLOCK>(mt);
     init_mixed_cols<BLOCK>(mixed_cols<BLOCK>());
   } else {
-    load_exp2_table();
+    load_fixed_tables(mt);
     load_math_tables();
   }
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_lsrk(const __grid_constant__ Me
     } else {
       while (!c.done) cell_attempt_full<V, SCH, BLOCK>(mt, c, p);
     }
-    cell_finish(mt, c);
+    cell_finish<V, BLOCK>(mt, c);
 #pragma unroll
     for (int k = 0; k < NSP; ++k) a.Y[k * a.ld + i] = c.X[k];
     a.T[i] = c.T;
@@ -74,21 +74,19 @@ __global__ void k_state_from_TPY(const __grid_constant__ MechTables mt, int64_t 
   e[i] = R_U * e_over_R(m, Ti);
 }
 
-// Launch with the mixed variant's dynamic shared memory (the per-thread columns).
+// Launch with the variant's dynamic shared memory (the per-thread columns).
 template <int V, int BLOCK, int MINB, int SCH>
 static cudaError_t launch_one(const MechTables &mt, const CellArgs &a, const StepParams &p, cudaStream_t s) {
-  size_t smem = 0;
-  if constexpr (V == CHEM_VARIANT_MIXED) {
-    smem = mixed_cols_bytes(BLOCK);
-    const cudaError_t e = allow_smem(reinterpret_cast<const void *>(k_lsrk<V, BLOCK, MINB, SCH>), smem);
-    if (e != cudaSuccess) return e;
-  }
+  const size_t smem = cols_bytes(V, BLOCK);
+  const cudaError_t e = allow_smem(reinterpret_cast<const void *>(k_lsrk<V, BLOCK, MINB, SCH>), smem);
+  if (e != cudaSuccess) return e;
   k_lsrk<V, BLOCK, MINB, SCH><<<(unsigned)((a.n + BLOCK - 1) / BLOCK), BLOCK, smem, s>>>(mt, a, p);
   return cudaGetLastError();
 }
 
-// The compiled shapes.  fp64: 12 warps per SM (128 x 3, 166 registers, no spills) or 16 (32, 64
-// threads, 128 registers).  The mixed two-register kernel's per-thread columns allow 16 warps
+// The compiled shapes.  fp64: 12 warps per SM (128 x 3, 168 registers, no spills) runs the
+// 1M-cell detonation slice in 30.5 ms, 16 (64 threads, 128 registers; its per-thread columns
+// and the tables leave 12) in 31.5, 32 threads in 34.9 and 8 warps (256) in 36.3.  The mixed two-register kernel's per-thread columns allow 16 warps
 // per SM (12 with 13 species): 128 x 4 at 128 registers, 7.9 ms on the 1M-cell detonation slice;
 // its 32- and 64-thread shapes keep 64 registers (14 warps of 64 threads, spilling): 9.3 ms at
 // 64, 11.2 at 32.

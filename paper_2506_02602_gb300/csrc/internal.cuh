@@ -64,10 +64,11 @@ struct BatchScratch {
   unsigned long long *cursor;    // [1] next queue slot
 };
 
-// Lets kernel fn use `bytes` of dynamic shared memory on the current device (needed above
-// 48 KB; set before each launch, as the setting is per device).
+// Lets kernel fn use `bytes` of dynamic shared memory on the current device (needed where they
+// and the static tables, under 24 KB, exceed 48 KB; set before each launch, as the setting is
+// per device).
 inline cudaError_t allow_smem(const void *fn, size_t bytes) {
-  return bytes <= 40 * 1024 ? cudaSuccess
+  return bytes <= 24 * 1024 ? cudaSuccess
                             : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 

@@ -66,6 +66,9 @@ struct MechTablesF32 {
   float T_mid2[2], ln_R_over_Pref2[2];
 };
 
+// A coefficient in fixed point: h 2^32 plus the top bits l of the lower half (2^2 l, or 2^4 l in qgt)
+struct QCoef { int32_t h, l; };
+
 // Per-context tables (host-built from chem_mechanism by build_tables()).
 struct MechTables {
   double T_mid;
@@ -87,12 +90,19 @@ struct MechTables {
   // fall-off low-pressure limit and Troe parameters (alpha, 1/T***, 1/T*, T**)
   double lnA0[NRX], beta0[NRX], Ta0[NRX];
   double troe_a[NRX], troe_i3[NRX], troe_i1[NRX], troe_T2[NRX];
-  // the same for the fixed-point exponentials (fastmath.cuh): log2 A (Q52), b (Q60),
-  // Ta / ln2 (Q46) of both limits, the Gibbs polynomials times -log2(e) and the Troe
-  // temperatures' factors times log2(e); fixed_ok: every coefficient is in their range
-  int64_t qA[NRX], qB[NRX], qH[NRX], qA0[NRX], qB0[NRX], qH0[NRX];
-  double gc_q[2][NSP][7];
+  // The fixed-point form's tables (rhs_fixed.cuh); fixed_ok: every coefficient is in its range.
+  // Rates: log2 A (Q52), b (Q58), -Ta / ln2 (Q46) of both limits; Troe temperatures' factors
+  // times log2(e).
+  int64_t qA[NRX], qA0[NRX];
+  QCoef qB[NRX], qH[NRX], qB0[NRX], qH0[NRX];
   double troe_q3[NRX], troe_q1[NRX], troe_q2[NRX];
+  // t = T 2^-S per range, S = q_log2[range]: ecw (Q37) times 2^(S (i+1)), the Gibbs functions
+  // times -log2(e) by log2 T (Q56), 1/T (Q44), t .. t^4 (Q57) and 1 (Q50)
+  QCoef qe[2][NSP][6];
+  QCoef qg[2][NSP][2], qgt[2][NSP][4];
+  int64_t qg1[2][NSP];
+  int64_t qT_mid, qRP;  // T_mid (Q50), log2(R_u / p_ref) (Q50)
+  int32_t q_log2[2];
   int32_t fixed_ok;
   // third-body efficiencies minus one: [M] = sum_k c_k + sum_k effm1 c_k
   double effm1[NRX][NSP];

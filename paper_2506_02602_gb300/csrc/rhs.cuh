@@ -5,28 +5,27 @@
 // reverse rates from equilibrium constants (Sec. 2.1.2), law of mass action (Eq. 16),
 // and F_k = W_k wdot_k / rho (Eq. 14, 20 at constant density).
 //
-// Arithmetic layout (an FP64 instruction occupies a warp's sub-partition for 64 cycles on
-// GB300, an integer one for 2, a wide multiply for 5; the FP64 pipe bounds the kernels):
-//   - exponentials run in fixed point on the integer pipe (exp2_q52, fastmath.cuh), the Arrhenius
-//     exponent with them: log2 A + b log2 T - (Ta / ln2) / T in 64-bit integers, no FP64
-//     instruction and at most 0.6 ulp off, for T in (128, 32768) K and coefficients within the
-//     forms' range; anything else takes the table-driven exp_t (production_rates_any).  The
-//     36 exponentials of an evaluation were 430 of its ~1040 FP64 instructions: with them gone
-//     the 1M-cell detonation slice takes 49.2 instead of 83.2 ms, a single warp's step 27 % less;
+// Two forms: nearly every evaluation takes rhs_fixed.cuh's, with its sums, exponentials and
+// logarithms in 64-bit fixed point on the integer pipe.  Here is the general form, for arguments
+// and coefficients outside that one's ranges (cell_rhs at the end chooses).
+//
+// Arithmetic layout of the general form (an FP64 instruction occupies a warp's sub-partition for
+// 64 cycles on GB300, so every fp64 operation counts):
+//   - exponentials and logarithms are the table-driven exp_t / log_t (fastmath.cuh);
 //   - g_k / RT comes from one combined NASA-7 polynomial per species (6 FMAs);
 //   - Newton works on mixture coefficients m_i = sum_k Y_k (ec_ki / W_k), assembled once
 //     per evaluation (54 FMAs), so each iteration is two Horner chains and a reciprocal;
 //   - equilibrium constants come from per-species G_k = exp(-g_k / RT):
 //     1/K_c,j = prod_reactants G * prod_products (1/G) * (R_u T / p_ref)^(sum nu), i.e.
-//     18 exponentials per evaluation (G and 1/G) instead of one per
+//     9 exponentials + 9 reciprocals per evaluation instead of one exponential per
 //     reaction; with a_k = c_k / G_k the net rate of progress is
 //     k_f (prod_reactants c - prod_reactants G * prod_products a * (R_u T / p_ref)^(sum nu)),
 //     one FMA for the reverse direction;
 //   - reciprocals are Newton-Raphson-refined hardware approximations (rcp1 / rcp2), ~3.5
 //     and ~5.7 FP64-pipe slots against ~9 for an IEEE divide; compares, clamps and
 //     fp32 <-> fp64 conversions run on the integer pipe (fastmath.cuh);
-//   - forward rates are one exponential per reaction (none for temperature-independent rates
-//     or A T^-1, A T^-2 with no activation).
+//   - forward rates are exp(ln A + beta ln T - Ta / T), one exponential per reaction
+//     (none for temperature-independent rates or A T^-1, A T^-2 with no activation).
 #pragma once
 
 #include <cmath>
@@ -34,6 +33,7 @@
 
 #include "fastmath.cuh"
 #include "mech.cuh"
+#include "rhs_fixed.cuh"
 
 namespace chem {
 
@@ -116,47 +116,32 @@ __device__ __forceinline__ bool solve_T(const MechTables &mt, const double (&Y)[
 // Quantities shared by every reaction of one evaluation.
 struct RateInputs {
   double lnT, invT, RTP, PRT, ctot;
-  long long lT, iT;  // log2 T (Q58), 1 / T (Q70): the fixed-point form's
-  double c[NSP];     // clamped concentrations, mol/m^3
-  double G[NSP];     // exp(-g_k / (R_u T))
-  double iG[NSP];    // c_k / G_k
+  double c[NSP];   // clamped concentrations, mol/m^3
+  double G[NSP];   // exp(-g_k / (R_u T))
+  double iG[NSP];  // c_k / G_k
 };
 
-// Temperatures of the fixed-point form: (128, 32768), on the high word.
-__device__ __forceinline__ bool fixed_range(double T) {
-  return (uint32_t)__double2hiint(T) - 0x40600001u < 0x40e00000u - 0x40600001u;
-}
-
 // Troe broadening factor (Gilbert, Luther & Troe 1983).
-template <int J, bool kFixed>
+template <int J>
 __device__ __forceinline__ double troe_F(const MechTables &mt, double T, double invT, double Pr) {
   constexpr int n = kRx[J].troe_n;
   if constexpr (n == 0) {
     return 1.0;
   } else {
     const double a = mt.troe_a[J];
-    double Fc;
-    if constexpr (kFixed) {
-      Fc = (1.0 - a) * exp2_lim(-T * mt.troe_q3[J]) + a * exp2_lim(-T * mt.troe_q1[J]);
-      if constexpr (n == 4) Fc += exp2_lim(-mt.troe_q2[J] * invT);
-    } else {
-      Fc = (1.0 - a) * exp_t(-T * mt.troe_i3[J]) + a * exp_t(-T * mt.troe_i1[J]);
-      if constexpr (n == 4) Fc += exp_t(-mt.troe_T2[J] * invT);
-    }
+    double Fc = (1.0 - a) * exp_t(-T * mt.troe_i3[J]) + a * exp_t(-T * mt.troe_i1[J]);
+    if constexpr (n == 4) Fc += exp_t(-mt.troe_T2[J] * invT);
     const double lFc = log10_t(Fc);
     const double cc = -0.4 - 0.67 * lFc;
     const double nn = 0.75 - 1.27 * lFc;
     const double x = log10_t(Pr) + cc;
     const double f1 = x * rcp2(nn - 0.14 * x);
-    const double lF = lFc * rcp2(1.0 + f1 * f1);
-    if constexpr (kFixed) return exp2_lim(lF * kLog2_10);
-    else return exp10_t(lF);
+    return exp10_t(lFc * rcp2(1.0 + f1 * f1));
   }
 }
 
-// Rate of progress of reaction J added into wdot (law of mass action, Eq. 16).  kFixed: the
-// exponentials in fixed point.
-template <int J, bool kFixed>
+// Rate of progress of reaction J added into wdot (law of mass action, Eq. 16).
+template <int J>
 __device__ __forceinline__ void reaction(const MechTables &mt, const RateInputs &in, double T,
                                          double (&wdot)[NSP]) {
   constexpr RxStruct R = kRx[J];
@@ -165,10 +150,8 @@ __device__ __forceinline__ void reaction(const MechTables &mt, const RateInputs 
   // kconst: 0 Arrhenius exponential; 1 constant (b = Ea = 0); 2, 3: A T^-1, A T^-2 (Ea = 0)
   const int kc = mt.kconst[J];
   double kf;
-  if (kc == 0) {
-    if constexpr (kFixed) kf = exp2_q52(limit_q52(arrhenius_log2(mt.qA[J], mt.qB[J], mt.qH[J], in.lT, in.iT)));
-    else kf = exp_t(fma(mt.beta[J], in.lnT, mt.lnA[J]) - mt.Ta[J] * in.invT);
-  } else if (kc == 1) kf = mt.A[J];
+  if (kc == 0) kf = exp_t(fma(mt.beta[J], in.lnT, mt.lnA[J]) - mt.Ta[J] * in.invT);
+  else if (kc == 1) kf = mt.A[J];
   else if (kc == 2) kf = mt.A[J] * in.invT;
   else kf = mt.A[J] * in.invT * in.invT;
   double M = 0.0;
@@ -181,11 +164,9 @@ __device__ __forceinline__ void reaction(const MechTables &mt, const RateInputs 
     }
   }
   if constexpr (R.type == FALLOFF) {
-    double k0;
-    if constexpr (kFixed) k0 = exp2_q52(limit_q52(arrhenius_log2(mt.qA0[J], mt.qB0[J], mt.qH0[J], in.lT, in.iT)));
-    else k0 = exp_t(fma(mt.beta0[J], in.lnT, mt.lnA0[J]) - mt.Ta0[J] * in.invT);
+    const double k0 = exp_t(fma(mt.beta0[J], in.lnT, mt.lnA0[J]) - mt.Ta0[J] * in.invT);
     const double Pr = k0 * M * rcp2(kf);
-    kf = (Pr > 0.0) ? kf * (Pr * rcp2(1.0 + Pr)) * troe_F<J, kFixed>(mt, T, in.invT, Pr) : 0.0;
+    kf = (Pr > 0.0) ? kf * (Pr * rcp2(1.0 + Pr)) * troe_F<J>(mt, T, in.invT, Pr) : 0.0;
   }
   // q = k_f (prod c_reactants - prod G_reactants prod (c / G)_products (R_u T / p)^dnu),
   // the same net rate as k_f prod c - k_r prod c with k_r = k_f / K_c
@@ -208,14 +189,13 @@ __device__ __forceinline__ void reaction(const MechTables &mt, const RateInputs 
   if constexpr (R.p1 >= 0) wdot[R.p1] += q;
 }
 
-template <bool kFixed, int... J>
+template <int... J>
 __device__ __forceinline__ void all_reactions(const MechTables &mt, const RateInputs &in, double T,
                                               double (&wdot)[NSP], std::integer_sequence<int, J...>) {
-  (reaction<J, kFixed>(mt, in, T, wdot), ...);
+  (reaction<J>(mt, in, T, wdot), ...);
 }
 
 // Molar production rates wdot (mol/m^3/s) at temperature T and clamped concentrations c.
-template <bool kFixed>
 __device__ __forceinline__ void production_rates(const MechTables &mt, double T,
                                                  const double (&c)[NSP], double (&wdot)[NSP]) {
   RateInputs in;
@@ -223,10 +203,6 @@ __device__ __forceinline__ void production_rates(const MechTables &mt, double T,
   in.invT = rcp2(T);
   in.RTP = (R_U / P_REF) * T;
   in.PRT = (P_REF / R_U) * in.invT;
-  if constexpr (kFixed) {
-    in.lT = (long long)abs_q<58>(in.lnT * kLog2E);
-    in.iT = (long long)abs_q<70>(in.invT);
-  }
   const double oml = 1.0 - in.lnT;
   const int range = ge_nonneg(T, mt.T_mid);
   double ctot = 0.0;
@@ -234,57 +210,52 @@ __device__ __forceinline__ void production_rates(const MechTables &mt, double T,
   for (int k = 0; k < NSP; ++k) {
     in.c[k] = c[k];
     ctot += c[k];
-    const double *gc = kFixed ? mt.gc_q[range][k] : mt.gc[range][k];
+    const double *gc = mt.gc[range][k];
     double g = fma(T, fma(T, fma(T, fma(T, gc[4], gc[3]), gc[2]), gc[1]), fma(gc[5], in.invT, gc[6]));
     g = fma(gc[0], oml, g);
-    // the limits keep G finite far outside the tables' range
-    if constexpr (kFixed) {
-      const long long y = to_q52(g);
-      in.G[k] = exp2_q52(y);
-      in.iG[k] = c[k] * exp2_q52(-y);
-    } else {
-      g = clamp_abs(g, 700.0);
-      in.G[k] = exp_t(-g);
-      in.iG[k] = c[k] * rcp2(in.G[k]);
-    }
+    g = clamp_abs(g, 700.0);  // keeps G finite far outside the tables' range
+    in.G[k] = exp_t(-g);
+    in.iG[k] = c[k] * rcp2(in.G[k]);
     wdot[k] = 0.0;
   }
   in.ctot = ctot;
-  all_reactions<kFixed>(mt, in, T, wdot, std::make_integer_sequence<int, NRX>{});
+  all_reactions(mt, in, T, wdot, std::make_integer_sequence<int, NRX>{});
 }
 
-// The form on exp_t, for temperatures or coefficients outside the fixed-point form's range;
-// out of line, as few evaluations come here.
-static __device__ __noinline__ void production_rates_any(const MechTables &mt, double T, const double *c,
-                                                         double *wdot) {
-  double cc[NSP], w[NSP];
+// dY/dt of one cell at fixed (rho, e) in the general form; out of line, as few evaluations come here.
+template <int ST>
+static __device__ __noinline__ bool cell_rhs_any(const MechTables &mt, const double *U, double rho, double invRho,
+                                                 double eR, double *T, double *F) {
+  double Y[NSP], c[NSP], wdot[NSP];
 #pragma unroll
-  for (int k = 0; k < NSP; ++k) cc[k] = c[k];
-  production_rates<false>(mt, T, cc, w);
-#pragma unroll
-  for (int k = 0; k < NSP; ++k) wdot[k] = w[k];
-}
-
-// dY/dt of one cell at fixed (rho, e).  T: in = Newton guess, out = solved T.
-// Returns false when the temperature solve fails.
-__device__ __forceinline__ bool cell_rhs(const MechTables &mt, const double (&Y)[NSP], double rho,
-                                         double invRho, double eR, double &T, double (&F)[NSP]) {
-  if (!solve_T(mt, Y, eR, T)) return false;
-  double c[NSP], wdot[NSP];
+  for (int k = 0; k < NSP; ++k) Y[k] = U[k * ST];
+  double Tn = *T;
+  const bool ok = solve_T(mt, Y, eR, Tn);
+  *T = Tn;
+  if (!ok) return false;
 #pragma unroll
   for (int k = 0; k < NSP; ++k) c[k] = clamp_nonneg(rho * (Y[k] * mt.invW[k]));
-  if (mt.fixed_ok && fixed_range(T)) {
-    production_rates<true>(mt, T, c, wdot);
-  } else {
-    double cc[NSP], w[NSP];
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) cc[k] = c[k];
-    production_rates_any(mt, T, cc, w);
-#pragma unroll
-    for (int k = 0; k < NSP; ++k) wdot[k] = w[k];
-  }
+  production_rates(mt, Tn, c, wdot);
 #pragma unroll
   for (int k = 0; k < NSP; ++k) F[k] = wdot[k] * mt.W[k] * invRho;
+  return true;
+}
+
+// dY/dt of one cell at fixed (rho, e) and the mass fractions in column U, which it overwrites.
+// T: in = Newton guess, out = solved T.  Returns false when the temperature solve fails.
+template <int ST>
+__device__ __forceinline__ bool cell_rhs(const MechTables &mt, const Fp64Cols &m, double rho,
+                                         double invRho, double eR, double &T, double (&F)[NSP]) {
+  if (mt.fixed_ok && fixed_rho(rho) && solve_T_fixed<ST>(mt, m.U, eR, T)) {
+    rates_fixed<ST>(mt, m, rho, T, F);
+    return true;
+  }
+  double Fc[NSP], Tc = T;
+  const bool ok = cell_rhs_any<ST>(mt, m.U, rho, invRho, eR, &Tc, Fc);
+  T = Tc;
+  if (!ok) return false;
+#pragma unroll
+  for (int k = 0; k < NSP; ++k) F[k] = Fc[k];
   return true;
 }
 

@@ -1,6 +1,6 @@
 """The fp64 right-hand side's fixed-point exponentials at the edges of their range.
 
-They serve temperatures in (128, 32768) K and coefficients that fit their fixed-point forms; any
+They serve temperatures in (128, 8192) K and coefficients that fit their fixed-point forms; any
 other evaluation takes the floating-point exponentials.  Cells on both sides of 128 K, and a
 mechanism with one coefficient beyond the forms' range (a temperature exponent of 8, its A
 scaled to the same rate at 1500 K), meet the oracle at the same bar as every fp64 cell: 1e-8
