@@ -195,6 +195,20 @@ int build_tables(const chem_mechanism *m, MechTables *t) {
       any |= t->effm1[j][k] != 0.0;
       mask |= (t->effm1[j][k] != 0.0) << k;
     }
+    if (kRx[j].type != ELEM) {
+      int n1 = 0, n0 = 0;
+      for (int k = 0; k < NSP; ++k) {
+        n1 += m->eff[j][k] != 1.0;
+        n0 += m->eff[j][k] != 0.0;
+      }
+      t->m_base[j] = n1 <= n0;
+      for (int k = 0; k < NSP; ++k) {
+        const double c = n1 <= n0 ? m->eff[j][k] - 1.0 : m->eff[j][k];
+        if (c == 0.0) continue;
+        t->m_k[j][t->m_n[j]] = (int8_t)k;
+        t->m_c[j][t->m_n[j]++] = c;
+      }
+    }
     t->has_eff[j] = any;
     t->eff_mask[j] = mask;
   }

@@ -189,13 +189,13 @@ __device__ __forceinline__ void cell_attempt_fp64(const MechTables &mt, CellStat
     c.done = true;
     return;
   }
-  // WRMS norm; the weights' reciprocals are Newton-Raphson-refined (two steps, within 2 ulp)
+  // WRMS norm; the weights' reciprocals are Newton-Raphson-refined (within 2 ulp)
   double sum = CUDART_NAN;
   if (!failed) {
     sum = 0.0;
 #pragma unroll kRoll
     for (int k = 0; k < NSP; ++k) {
-      const double w = m.E[k * ST] * rcp2(fma(p.rtol, max_abs(c.X[k], m.X[k * ST]), p.atol));
+      const double w = m.E[k * ST] * rcp3(fma(p.rtol, max_abs(c.X[k], m.X[k * ST]), p.atol));
       sum = fma(w, w, sum);
     }
   }

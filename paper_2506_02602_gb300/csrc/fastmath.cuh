@@ -76,18 +76,21 @@ __device__ __forceinline__ double clamp_abs(double x, double lim) {
 }
 
 // ---- exponentials in fixed point, on the integer pipe ----
-// A 64-bit number in units of 2^-52 (Q52) stands for a base-2 logarithm: its 1/1024ths index
-// a table of 64-bit mantissas (8 KB in shared memory), and 2^r - 1 for the rest, r < 2^-10,
-// is u + u^2/2 in integer arithmetic with u = r ln2 (r in units of 2^-74) and the terms from
-// u^3 on in fp32.  No FP64 instruction: about 60 integer and wide-multiply instructions, 140
-// cycles of a sub-partition on GB300 against 640 for the table-driven exp_t, and at most
-// 0.6 ulp off.
+// A 64-bit number in units of 2^-52 (Q52) stands for a base-2 logarithm.  Its first two tens of
+// fraction bits index tables (8 KB each in shared memory) of 2^(j/2^10) and 2^(k/2^20) - 1, and
+// the last 32, r < 2^-20, give 2^r - 1 as v + v^2/2 with v = r ln2.  No FP64 instruction, two wide
+// and five high multiplies, and at most 0.51 ulp off: 32 instructions.
+// (With one table and r < 2^-10 the terms to r^4, half of them in fp32, and their alignment took
+// about twice as many.)
 
-// Per-block copy of k_exp2_q63, filled by load_exp2_table().
-__shared__ unsigned long long s_exp2_q63[1024];
+// Per-block copies of k_exp2_hi and k_exp2_lo, filled by load_exp2_tables().
+__shared__ unsigned long long s_exp2_hi[1024], s_exp2_lo[1024];
 
-__device__ __forceinline__ void load_exp2_table() {
-  for (int i = threadIdx.x; i < 1024; i += blockDim.x) s_exp2_q63[i] = k_exp2_q63[i];
+__device__ __forceinline__ void load_exp2_tables() {
+  for (int i = threadIdx.x; i < 1024; i += blockDim.x) {
+    s_exp2_hi[i] = k_exp2_hi[i];
+    s_exp2_lo[i] = k_exp2_lo[i];
+  }
   __syncthreads();
 }
 
@@ -95,20 +98,17 @@ __device__ __forceinline__ unsigned long long mul_wide(uint32_t a, uint32_t b) {
 
 // 2^(y 2^-52) for |y| < 1021 2^52
 __device__ __forceinline__ double exp2_q52_body(long long y) {
-  const uint32_t yl = (uint32_t)y;
-  const int yh = (int)(y >> 32), k = yh >> 10;
-  const uint32_t fh = __funnelshift_l(yl, (uint32_t)yh, 22), fl = yl << 22;  // r in units of 2^-74
-  const unsigned long long u = mul_wide(fh, kLn2Q64Hi) + __umulhi(fh, kLn2Q64Lo) + __umulhi(fl, kLn2Q64Hi);
-  const uint32_t uh = (uint32_t)(u >> 32), ul = (uint32_t)u;
-  const unsigned long long u2 = (mul_wide(uh, uh) >> 1) + __umulhi(uh, ul);  // u^2 / 2, units of 2^-84
-  const float g = (float)uh * 0x1p-42f;
-  const uint32_t c = (uint32_t)(g * g * g * fmaf(g, 0x1p64f / 24.0f, 0x1p64f / 6.0f));  // u^3/6 + u^4/24, 2^-64
-  const unsigned long long p = u + (u2 >> 10) + ((unsigned long long)c << 10);          // 2^r - 1, 2^-74
-  const unsigned long long t = s_exp2_q63[k & 1023];
-  const uint32_t th = (uint32_t)(t >> 32), tl = (uint32_t)t, ph = (uint32_t)(p >> 32), pl = (uint32_t)p;
-  const unsigned long long tp = mul_wide(th, ph) + __umulhi(th, pl) + __umulhi(tl, ph);  // 2^-73
-  const unsigned long long m = (t + (tp >> 10) + 0x400ull) >> 11;  // 53 bits, rounded; carries into the exponent
-  return __longlong_as_double((long long)((unsigned long long)(uint32_t)((k >> 10) + 1022) << 52) + (long long)m);
+  const uint32_t yl = (uint32_t)y, yh = (uint32_t)(y >> 32);
+  const unsigned long long t = s_exp2_hi[(yh >> 10) & 1023], s0 = s_exp2_lo[yh & 1023];
+  const unsigned long long v = mul_wide(yl, kLn2Q64Hi) + __umulhi(yl, kLn2Q64Lo);  // units of 2^-84
+  const uint32_t vh = (uint32_t)(v >> 32);
+  const unsigned long long w = v + mul_wide(__umulhi(vh, vh), 2048u);  // + v^2/2
+  // (1 + s0) (1 + w) - 1 in units of 2^-64
+  const unsigned long long s = s0 + (w >> 20) + mul_wide(__umulhi((uint32_t)(s0 >> 22), (uint32_t)(w >> 32)), 4u);
+  const uint32_t th = (uint32_t)(t >> 32), tl = (uint32_t)t, sh = (uint32_t)(s >> 32), sl = (uint32_t)s;
+  const unsigned long long p = (t + mul_wide(th, sh) + __umulhi(th, sl) + __umulhi(tl, sh)) >> 11;  // 53 bits, rounded
+  // the leading bit, or a carry, adds to the exponent
+  return __hiloint2double((int)((uint32_t)(p >> 32) + (yh & 0xfff00000u) + (1022u << 20)), (int)(uint32_t)p);
 }
 
 // Out of line, as exp_t: one copy of the code; two at a time where there are two, whose chains
@@ -131,6 +131,13 @@ __device__ __forceinline__ unsigned long long abs_q(double x) {
 __device__ __forceinline__ long long to_q52(double x) {
   const long long v = (long long)abs_q<52>(clamp_abs(x, 1009.875));
   return __double2hiint(x) < 0 ? -v : v;
+}
+
+// x in units of 2^-Q kept within +-1020 by its upper word
+template <int Q>
+__device__ __forceinline__ long long limit_q(long long x) {
+  const int lim = 1019 << (Q - 32), h = min(max((int)(x >> 32), -lim), lim);
+  return (long long)(((unsigned long long)(uint32_t)h << 32) | (uint32_t)x);
 }
 
 // ---- sums of products in fixed point ----
@@ -174,20 +181,33 @@ __device__ __forceinline__ void load_log2_table() {
   __syncthreads();
 }
 
-// log2 x in units of 2^-58 for positive normal x, at most 8 units off: x = 2^e f, r = f c_j - 1
-// exact in units of 2^-67 (|r| < 2^-8.9), log2(1 + r) with the terms from r^4 on in fp32.
-static __device__ __noinline__ long long log2_q58(double x) {
+// log2 x = e + f, f in units of 2^-58, for positive normal x, at most 6 units off: x = 2^e (1 + ..),
+// r = x 2^-e c_j - 1 exact in units of 2^-71 (|r| < 2^-8.9), log2(1 + r) with the terms from r^4
+// on in fp32.
+__device__ __forceinline__ long long log2_parts(double x, int &e) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int e = (int)(b >> 52) - 1023, j = (int)(b >> 44) & 255;
+  e = (int)(b >> 52) - 1023;
+  const int j = (int)(b >> 44) & 255;
   const unsigned long long f = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
-  const long long r = (long long)((f * s_log2_c[j]) << 4);  // units of 2^-71; the 1 drops out
+  const long long r = (long long)((f * s_log2_c[j]) << 4);    // the 1 drops out
   const long long u = __mul64hi(r, kLog2E_q62);               // r log2(e), 2^-69
   const long long r2 = __mul64hi(r, r);                       // r^2, 2^-78
   const long long t = __mul64hi(r2, kLog2E_q62);              // r^2 log2(e) / 2, 2^-77
   const long long c = __mul64hi(__mul64hi(r2, r), kLog2EThird_q64);  // r^3 log2(e) / 3, 2^-85
   const float rf = (float)(int)(r >> 32) * 0x1p-39f, rf2 = rf * rf;
   const float d = rf2 * rf2 * (0x1p58f * (float)kLog2E) * fmaf(rf, 0.2f, -0.25f);
-  return ((long long)e << 58) + s_log2_q58[j] + (u >> 11) - (t >> 19) + (c >> 27) + (long long)(int)d;
+  return s_log2_q58[j] + (u >> 11) - (t >> 19) + (c >> 27) + (long long)(int)d;
+}
+// In units of 2^-58 for x in (2^-31, 2^31), and in units of 2^-52 for any positive normal x.
+__device__ __forceinline__ long long log2_q58(double x) {
+  int e;
+  const long long f = log2_parts(x, e);
+  return ((long long)e << 58) + f;
+}
+static __device__ __noinline__ long long log2_q52(double x) {
+  int e;
+  const long long f = log2_parts(x, e);
+  return ((long long)e << 52) + (f >> 6);
 }
 
 // x 2^-50 for x in (2^57, 2^63)
@@ -197,10 +217,6 @@ __device__ __forceinline__ double q50_to_double(long long x) {
   return __longlong_as_double(((long long)(1035 - n) << 52) + (long long)m);  // the leading one adds to the exponent
 }
 
-__device__ __forceinline__ long long limit_q52(long long y) {
-  const long long lim = 1019ll << 52;
-  return min(max(y, -lim), lim);
-}
 
 // log(x) for positive normal finite x.
 __device__ __forceinline__ double log_tab(double x) {
@@ -287,6 +303,13 @@ __device__ __forceinline__ double rcp1(double x) {
 __device__ __forceinline__ double rcp2(double x) {
   const double r = rcp1(x);
   return fma(r, fma(-x, r, 1.0), r);
+}
+// as close as rcp2 in one third-order step, r (1 + d + d^2) with d = 1 - x r: three FP64
+// instructions instead of four
+__device__ __forceinline__ double rcp3(double x) {
+  const double r = rcp_approx(x);
+  const double d = fma(-x, r, 1.0);
+  return fma(r, fma(d, d, d), r);
 }
 
 // ---- fp64 tests and selects on the integer pipe ----

@@ -4,7 +4,8 @@ exp (Tang 1989, "Table-driven implementation of the exponential function in IEEE
 floating-point arithmetic"): x = (128 m + j) ln2/128 + r, exp(x) = 2^m 2^(j/128) e^r with
 |r| <= ln2/256; the table holds 2^(j/128), j = 0..127, each correctly rounded.
 
-exp2 in fixed point (exp2_q52): 2^(j/1024), j = 0..1023, rounded to 64-bit integers in units of 2^-63.
+exp2 in fixed point (exp2_q52): 2^(j/2^10) and 2^(j/2^20) - 1, j = 0..1023, rounded to 64-bit
+integers in units of 2^-63 and 2^-64.
 
 log2 in fixed point (log2_q58): c_j = 2^15 / (1 + (j + 1/2) / 256), j = 0..255, rounded to
 integers, and -log2(c_j 2^-15) of the rounded c_j in units of 2^-58.
@@ -50,11 +51,17 @@ def main():
     for j in range(128):
         out.append(f"    {hexd((Decimal(j) / 128 * LN2).exp())},")
     out.append("};")
-    out.append("// 2^(j/1024) in units of 2^-63, j = 0..1023")
-    out.append("__device__ const unsigned long long k_exp2_q63[1024] = {")
+    out.append("// 2^(j/2^10) in units of 2^-63 plus half a unit of a 53-bit mantissa, j = 0..1023")
+    out.append("__device__ const unsigned long long k_exp2_hi[1024] = {")
     for j in range(1024):
-        v = int(((Decimal(j) / 1024 * LN2).exp() * 2**63).to_integral_value())
+        v = int(((Decimal(j) / 1024 * LN2).exp() * 2**63).to_integral_value()) + 1024
         out.append(f"    {v:#018x}ull,")
+    out.append("};")
+    out.append("// 2^(j/2^20) - 1 in units of 2^-64, j = 0..1023")
+    out.append("__device__ const unsigned long long k_exp2_lo[1024] = {")
+    for j in range(1024):
+        v = int((((Decimal(j) / 2**20 * LN2).exp() - 1) * 2**64).to_integral_value())
+        out.append(f"    {v:#016x}ull,")
     out.append("};")
     cq = [int((2**15 / (1 + (j + Decimal(1) / 2) / 256)).to_integral_value()) for j in range(256)]
     out.append("// c_j = RN(2^15 / (1 + (j + 1/2) / 256)), j = 0..255")

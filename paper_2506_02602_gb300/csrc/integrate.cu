@@ -85,8 +85,8 @@ static cudaError_t launch_one(const MechTables &mt, const CellArgs &a, const Ste
 }
 
 // The compiled shapes.  fp64: 12 warps per SM (128 x 3, 168 registers, no spills) runs the
-// 1M-cell detonation slice in 30.5 ms, 16 (64 threads, 128 registers; its per-thread columns
-// and the tables leave 12) in 31.5, 32 threads in 34.9 and 8 warps (256) in 36.3.  The mixed two-register kernel's per-thread columns allow 16 warps
+// 1M-cell detonation slice in 26.1 ms, 64 threads (128 registers; the columns and the 23 KB of
+// tables leave 10 warps) in 28.6, 32 threads in 37.1 and 8 warps (256) in 31.7.  The mixed two-register kernel's per-thread columns allow 16 warps
 // per SM (12 with 13 species): 128 x 4 at 128 registers, 7.9 ms on the 1M-cell detonation slice;
 // its 32- and 64-thread shapes keep 64 registers (14 warps of 64 threads, spilling): 9.3 ms at
 // 64, 11.2 at 32.

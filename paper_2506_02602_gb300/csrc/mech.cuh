@@ -108,6 +108,11 @@ struct MechTables {
   double effm1[NRX][NSP];
   int32_t has_eff[NRX];
   int32_t eff_mask[NRX];  // bit k set where effm1[j][k] != 0 (the fp64 sums skip the rest)
+  // the same as short lists: [M] = m_base sum_k c_k + sum_i m_c[i] c[m_k[i]], m_base 1 or 0,
+  // whichever makes the shorter list of m_n entries
+  double m_c[NRX][NSP];
+  int32_t m_base[NRX], m_n[NRX];
+  int8_t m_k[NRX][NSP];
   double ln_R_over_Pref;  // ln(R_u / p_ref): ln(R_u T / p_ref) = ln T + this
   // Newton's quadratic-convergence stop: after a step dT the remaining error is at most
   // (C / 2) dT^2 with C = max |c_v' / c_v| of the tables on [200, 6000] K, so a step with

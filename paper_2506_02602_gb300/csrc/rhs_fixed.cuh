@@ -16,9 +16,9 @@
 //     progress is k_f (prod y_reactants - K prod y_products): 4 FP64 instructions, and reactions
 //     of one stoichiometry (duplicates, colliders) share it with their k_f summed.
 // A warp's evaluation issued 1040 FP64 instructions in the general form, 637 with only its
-// exponentials in fixed point and 350 here; the 1M-cell detonation slice takes 83.2, 49.2 and
-// 30.5 ms, a 256-cell batch of 15 steps 3.0, 2.1 and 1.7 ms (one warp's chain of dependent
-// instructions).  Integer work now fills the issue slots the FP64 pipe (75 % busy) leaves.
+// exponentials in fixed point and 300 here; the 1M-cell detonation slice takes 83.2, 49.2 and
+// 26.1 ms, a 256-cell batch of 15 steps 3.0, 2.1 and 1.5 ms (one warp's chain of dependent
+// instructions).  Integer work now fills the issue slots the FP64 pipe (70 % busy) leaves.
 //
 // For T in (128, 8192) K, |Y_k| < 1.25, rho in (2^-64, 2^64) and coefficients within the
 // tables' ranges (MechTables::fixed_ok); anything else takes the general form (rhs.cuh).
@@ -59,7 +59,7 @@ __shared__ int4 s_qg[2][NSP][4];
 
 __device__ __forceinline__ int4 pack_q(const QCoef &a, const QCoef &b) { return make_int4(a.h, a.l, b.h, b.l); }
 __device__ __forceinline__ void load_fixed_tables(const MechTables &mt) {
-  load_exp2_table();
+  load_exp2_tables();
   load_log2_table();
   for (int i = threadIdx.x; i < 2 * NSP; i += blockDim.x) {
     const int r = i / NSP, k = i % NSP;
@@ -151,13 +151,14 @@ struct RateInputsQ {
   double T, invT, ctot;
   Limbs<2> lT, iT;       // log2 T (Q58), 1/T (Q70)
   long long lrho, lRT;   // log2 rho (Q52), log2(rho R_u T / p_ref) (Q50)
-  double y[NSP];         // Y_k / W_k, clamped
+  const double *U;       // column of Y_k / W_k, clamped
+  double y[NSP];         // the same
   long long g[NSP];      // -g_k / (R_u T ln2) (Q50)
 };
 
 // log2 x; zero, negative, subnormal and non-finite arguments by the library
 __device__ __forceinline__ double log2_any(double x) {
-  if (pos_normal(x)) return (double)log2_q58(x) * 0x1p-58;
+  if (pos_normal(x)) return (double)log2_q52(x) * 0x1p-52;
   return log(x) * kLog2E;
 }
 
@@ -170,23 +171,23 @@ __device__ __forceinline__ long long rate_log2(int64_t a, const QCoef &b, const 
   return s.value();
 }
 
+// Third-body sums [M] / rho go through the list of efficiencies that differ from the base, 1 or 0,
+// a rolled loop of a few entries: unrolled over all species under their mask, the compiler
+// computed every term and selected, 41 FP64 instructions a warp more.
 // Forward rate coefficient of reaction J times rho^(order - 1), third body and fall-off included:
 // in the units of y.  With kK also K = 2^lK, whose exponential joins one of the rate's.
-template <int J, bool kK>
+template <int ST, int J, bool kK>
 __device__ __forceinline__ double rate_fixed(const MechTables &mt, const RateInputsQ &in, long long lK, double &K) {
   constexpr RxStruct R = kRx[J];
   constexpr int pw = n_reac(R) - 1;
   double M = 0.0;
   if constexpr (R.type != ELEM) {
-    M = in.ctot;
-    if (mt.has_eff[J]) {
-#pragma unroll
-      for (int k = 0; k < NSP; ++k)
-        if ((mt.eff_mask[J] >> k) & 1) M = fma(mt.effm1[J][k], in.y[k], M);
-    }
+    M = mt.m_base[J] ? in.ctot : 0.0;
+#pragma unroll 1
+    for (int i = 0; i < mt.m_n[J]; ++i) M = fma(mt.m_c[J][i], in.U[mt.m_k[J][i] * ST], M);
   }
   if constexpr (R.type != FALLOFF) {
-    const long long l = limit_q52(rate_log2<pw + (R.type == THIRD_BODY)>(mt.qA[J], mt.qB[J], mt.qH[J], in));
+    const long long l = limit_q<52>(rate_log2<pw + (R.type == THIRD_BODY)>(mt.qA[J], mt.qB[J], mt.qH[J], in));
     double kf;
     if constexpr (kK) {
       const double2 v = exp2_q52(l, lK);
@@ -199,10 +200,10 @@ __device__ __forceinline__ double rate_fixed(const MechTables &mt, const RateInp
   } else {
     const long long li = rate_log2<pw>(mt.qA[J], mt.qB[J], mt.qH[J], in);
     const long long l0 = rate_log2<pw + 1>(mt.qA0[J], mt.qB0[J], mt.qH0[J], in);
-    const double2 v = exp2_q52(limit_q52(li), limit_q52(l0));
+    const double2 v = exp2_q52(limit_q<52>(li), limit_q<52>(l0));
     const double k0M = v.y * M;
     // k_inf Pr / (1 + Pr), Pr = k0 M / k_inf
-    double kf = k0M > 0.0 ? v.x * (k0M * rcp2(v.x + k0M)) : 0.0;
+    double kf = k0M > 0.0 ? v.x * (k0M * rcp3(v.x + k0M)) : 0.0;
     if constexpr (R.troe_n != 0) {
       // Troe broadening (Gilbert, Luther & Troe 1983) in log2: with x = lg Pr - 0.4 - 0.67 lg Fc and
       // d = 0.75 - 1.27 lg Fc - 0.14 x, log F = log Fc d^2 / (d^2 + x^2)
@@ -219,7 +220,7 @@ __device__ __forceinline__ double rate_fixed(const MechTables &mt, const RateInp
       const double x = fma(-0.67, lFc, lPr - 0.4 * kLog2_10);
       const double d = fma(-0.14, x, fma(-1.27, lFc, 0.75 * kLog2_10));
       const double d2 = d * d;
-      const long long lF = to_q52(lFc * (d2 * rcp2(fma(x, x, d2))));
+      const long long lF = to_q52(lFc * (d2 * rcp3(fma(x, x, d2))));
       double F;
       if constexpr (kK && R.troe_n != 4) {
         const double2 w = exp2_q52(lF, lK);
@@ -276,18 +277,18 @@ __device__ __forceinline__ void rate_add(double q, double (&wdot)[NSP]) {
   else wdot[K] = fma((double)NU, q, wdot[K]);
 }
 
-template <int J, int I>
+template <int ST, int J, int I>
 __device__ __forceinline__ void rate_member(const MechTables &mt, const RateInputsQ &in, double &kF, double &kR) {
   if constexpr (I != J && rx_leader(I) == J) {
     double none;
-    const double k = rate_fixed<I, false>(mt, in, 0, none);
+    const double k = rate_fixed<ST, I, false>(mt, in, 0, none);
     kF += k;
     if (mt.reversible[I]) kR += k;
   }
 }
 
 // Net rate of progress of the reactions of J's stoichiometry into wdot, J the first of them
-template <int J, int... I>
+template <int ST, int J, int... I>
 __device__ __forceinline__ void reaction_fixed(const MechTables &mt, const RateInputsQ &in, double (&wdot)[NSP],
                                                std::integer_sequence<int, I...>) {
   if constexpr (rx_leader(J) == J) {
@@ -297,16 +298,15 @@ __device__ __forceinline__ void reaction_fixed(const MechTables &mt, const RateI
     long long l = in.g[R.r0] - in.g[R.p0] + dnu * in.lRT;
     if constexpr (R.r1 >= 0) l += in.g[R.r1];
     if constexpr (R.p1 >= 0) l -= in.g[R.p1];
-    const long long lim = 1019ll << 50;
     double K;
-    double kF = rate_fixed<J, true>(mt, in, min(max(l, -lim), lim) << 2, K);
+    double kF = rate_fixed<ST, J, true>(mt, in, limit_q<50>(l) << 2, K);
     double yr = in.y[R.r0], yp = in.y[R.p0];
     if constexpr (R.r1 >= 0) yr *= in.y[R.r1];
     if constexpr (R.p1 >= 0) yp *= in.y[R.p1];
     double q;
     if constexpr (rx_group(J) > 1) {
       double kR = mt.reversible[J] ? kF : 0.0;
-      (rate_member<J, I>(mt, in, kF, kR), ...);
+      (rate_member<ST, J, I>(mt, in, kF, kR), ...);
       q = fma(kF, yr, -(kR * (K * yp)));
     } else {
       q = kF * (mt.reversible[J] ? fma(-K, yp, yr) : yr);
@@ -326,10 +326,10 @@ __device__ __forceinline__ void reaction_fixed(const MechTables &mt, const RateI
   }
 }
 
-template <int... J>
+template <int ST, int... J>
 __device__ __forceinline__ void all_reactions_fixed(const MechTables &mt, const RateInputsQ &in, double (&wdot)[NSP],
                                                     std::integer_sequence<int, J...> seq) {
-  (reaction_fixed<J>(mt, in, wdot, seq), ...);
+  (reaction_fixed<ST, J>(mt, in, wdot, seq), ...);
 }
 
 // dY/dt at T from solve_T_fixed; U becomes the concentrations per mass.
@@ -337,12 +337,13 @@ template <int ST>
 __device__ __forceinline__ void rates_fixed(const MechTables &mt, const Fp64Cols &m, double rho, double T,
                                             double (&F)[NSP]) {
   RateInputsQ in;
+  in.U = m.U;
   in.T = T;
-  in.invT = rcp2(T);
+  in.invT = rcp3(T);
   const long long lT = log2_q58(T);
   in.lT = limbs<2>(lT);
   in.iT = limbs<2>((long long)abs_q<70>(in.invT));
-  in.lrho = log2_q58(rho) >> 6;
+  in.lrho = log2_q52(rho);
   in.lRT = (lT >> 8) + mt.qRP + (in.lrho >> 2);
   {
     const int range = ge_nonneg(T, mt.T_mid);
@@ -373,7 +374,7 @@ __device__ __forceinline__ void rates_fixed(const MechTables &mt, const Fp64Cols
     in.g[k] = m.g[k * ST];
   }
   double wdot[NSP];
-  all_reactions_fixed(mt, in, wdot, std::make_integer_sequence<int, NRX>{});
+  all_reactions_fixed<ST>(mt, in, wdot, std::make_integer_sequence<int, NRX>{});
 #pragma unroll
   for (int k = 0; k < NSP; ++k) F[k] = ((kReactive >> k) & 1) ? wdot[k] * mt.W[k] : 0.0;
 }
