@@ -14,11 +14,13 @@
 namespace chem {
 
 // MSE over the first `nout` columns: loss += sum (y - t)^2 / (M nout); dY = 2 (y - t) / (M nout)
-// (bf16, padded columns zero).  loss is accumulated with one atomic per block.
+// (bf16, padded columns zero).  loss is accumulated with one atomic per block.  A captured
+// training step's counter advances here, between the kernels that read it.
 __global__ void k_mse(int64_t M, int nout, int ldy, const float *__restrict__ Y,
                       const float *__restrict__ Tg, int ldt, __nv_bfloat16 *__restrict__ dY,
-                      int lddy, float *loss) {
+                      int lddy, float *loss, int64_t *step) {
   __shared__ float red[256];
+  if (step && blockIdx.x == 0 && threadIdx.x == 0) *step += 1;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   float l = 0.0f;
   if (idx < M * lddy) {
@@ -40,25 +42,31 @@ __global__ void k_mse(int64_t M, int nout, int ldy, const float *__restrict__ Y,
   if (threadIdx.x == 0) atomicAdd(loss, red[0] / (float)(M * nout));
 }
 
-// db[n] = sum_m dZ[m, n] (one block per 32 columns, fp32 accumulation)
-// Partial column sums: CTA (x, y) sums rows y, y + nsplit, ... of columns 32x .. 32x+31
-// into part[y * N + n] (8 row groups per CTA, combined in a fixed order).
-__global__ void k_bias_grad(int64_t M, int N, const __nv_bfloat16 *__restrict__ dZ, int ld,
-                            float *__restrict__ part) {
+// Partial column sums of dZ [M x N], all layers in one launch: CTA (x, y) sums rows y, y + nsplit,
+// ... of a layer's columns 32 x' .. 32 x' + 31 into part[l][y * N + n] (8 row groups per CTA,
+// combined in a fixed order).  Latency-bound: eight loads in flight a thread, and all layers
+// take 6.2 us at 4096 rows where four launches and their reductions took 11 each.
+__global__ void k_bias_grad(int64_t M, const __grid_constant__ BiasSegs sg) {
   __shared__ float red[8][33];
-  const int n = blockIdx.x * 32 + (threadIdx.x & 31);
+  int l = 0, x = blockIdx.x;
+  while (x >= (sg.N[l] + 31) / 32) x -= (sg.N[l++] + 31) / 32;
+  const int N = sg.N[l];
+  const __nv_bfloat16 *__restrict__ dZ = sg.dZ[l];
+  const int n = x * 32 + (threadIdx.x & 31);
   const int row = threadIdx.x >> 5;  // 8 row groups
   const int64_t stride = 8 * (int64_t)gridDim.y;
   float s = 0.0f;
-  if (n < N)
-    for (int64_t m = (int64_t)blockIdx.y * 8 + row; m < M; m += stride) s += __bfloat162float(dZ[m * ld + n]);
+  if (n < N) {
+#pragma unroll 8
+    for (int64_t m = (int64_t)blockIdx.y * 8 + row; m < M; m += stride) s += __bfloat162float(dZ[m * N + n]);
+  }
   red[row][threadIdx.x & 31] = s;
   __syncthreads();
   if (threadIdx.x < 32 && n < N) {
     float t = 0.0f;
 #pragma unroll
     for (int r = 0; r < 8; ++r) t += red[r][threadIdx.x];
-    part[(int64_t)blockIdx.y * N + n] = t;
+    sg.part[l][(int64_t)blockIdx.y * N + n] = t;
   }
 }
 
@@ -93,11 +101,12 @@ __global__ void k_adam(int64_t n, float *__restrict__ w, const float *__restrict
   }
 }
 
-// Adam on every parameter (the segments of AdamSegs) with the step's learning rate and
+// The gradient's split partial sums added in order of the split (as k_reduce_splits) and Adam on
+// every parameter (the segments of AdamSegs) with the step's learning rate and
 // bias corrections read from a device schedule: sched[3 t .. 3 t + 2] = {lr, 1 - b1^(t+1),
-// 1 - b2^(t+1)} at t = *step (a CUDA graph of one training step replays with the counter
-// advancing on the device).
-__global__ void k_adam_sched_all(int64_t n, float *__restrict__ w, const float *__restrict__ g,
+// 1 - b2^(t+1)} at t = *step - 1 (a CUDA graph of one training step replays with the counter
+// advancing on the device).  The eight reductions were launches of their own, 3.5 us each.
+__global__ void k_adam_sched_all(int64_t n, float *__restrict__ w,
                                  float *__restrict__ m, float *__restrict__ v, const float *__restrict__ sched,
                                  const int64_t *__restrict__ step, float b1, float b2, float eps,
                                  const __grid_constant__ AdamSegs sg) {
@@ -105,10 +114,13 @@ __global__ void k_adam_sched_all(int64_t n, float *__restrict__ w, const float *
   if (i >= n) return;
   int j = 0;
   while (j < kAdamSegs - 1 && i >= sg.end[j]) ++j;
-  const int64_t li = i - (j ? sg.end[j - 1] : 0);
-  const float *sc = sched + 3 * *step;
+  const int64_t base = j ? sg.end[j - 1] : 0, li = i - base, len = sg.end[j] - base;
+  const float *sc = sched + 3 * (*step - 1);
   const float lr = sc[0], bc1 = sc[1], bc2 = sc[2];
-  const float gi = g[i];
+  const float *part = sg.part[j] + li;
+  float gi = 0.0f;
+#pragma unroll 16
+  for (int z = 0; z < sg.nsplit; ++z) gi += part[z * len];
   const float mi = b1 * m[i] + (1.0f - b1) * gi;
   const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
   m[i] = mi;
@@ -122,21 +134,18 @@ __global__ void k_adam_sched_all(int64_t n, float *__restrict__ w, const float *
   }
 }
 
-// out[r, :] = in[idx[base + r], :] with base = (*step mod nbatch) * nrows: the batch of
-// the current step of an epoch's permutation
-__global__ void k_gather_rows_step(int64_t nrows, int ncol, const int32_t *__restrict__ idx,
-                                   const int64_t *__restrict__ step, int64_t nbatch, const float *__restrict__ in,
-                                   int ldin, float *__restrict__ out, int ldout) {
+// The batch of step *step of an epoch's permutation, rows idx[base + r] with base = (*step mod
+// nbatch) * nrows: features as bf16 and targets, ncol columns each
+__global__ void k_gather_batch(int64_t nrows, int ncol, const int32_t *__restrict__ idx,
+                               const int64_t *__restrict__ step, int64_t nbatch, const float *__restrict__ X,
+                               const float *__restrict__ T, __nv_bfloat16 *__restrict__ Xb, float *__restrict__ Tb) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nrows * ncol) return;
   const int64_t r = t / ncol;
   const int c = (int)(t % ncol);
-  const int64_t base = (*step % nbatch) * nrows;
-  out[r * ldout + c] = in[(int64_t)idx[base + r] * ldin + c];
-}
-
-__global__ void k_step_inc(int64_t *step) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) *step += 1;
+  const int64_t from = (int64_t)idx[(*step % nbatch) * nrows + r] * ncol + c;
+  Xb[t] = __float2bfloat16(X[from]);
+  Tb[t] = T[from];
 }
 
 // bf16 copy of a float matrix (for the gathered input features)
@@ -148,8 +157,8 @@ __global__ void k_to_bf16(int64_t n, const float *__restrict__ in, __nv_bfloat16
 static unsigned blocks(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
 cudaError_t launch_mse(int64_t M, int nout, int ldy, const float *Y, const float *Tg, int ldt,
-                       __nv_bfloat16 *dY, int lddy, float *loss, cudaStream_t s) {
-  k_mse<<<blocks(M * lddy, 256), 256, 0, s>>>(M, nout, ldy, Y, Tg, ldt, dY, lddy, loss);
+                       __nv_bfloat16 *dY, int lddy, float *loss, int64_t *step, cudaStream_t s) {
+  k_mse<<<blocks(M * lddy, 256), 256, 0, s>>>(M, nout, ldy, Y, Tg, ldt, dY, lddy, loss, step);
   return cudaGetLastError();
 }
 cudaError_t launch_reduce_splits(int64_t n, int nsplit, const float *part, int64_t split_ld, float *out,
@@ -158,11 +167,11 @@ cudaError_t launch_reduce_splits(int64_t n, int nsplit, const float *part, int64
   k_reduce_splits<<<blocks(n, 256), 256, 0, s>>>(n, nsplit, part, split_ld, out);
   return cudaGetLastError();
 }
-cudaError_t launch_bias_grad(int64_t M, int N, const __nv_bfloat16 *dZ, int ld, float *part, int nsplit,
-                             float *db, cudaStream_t s) {
-  k_bias_grad<<<dim3(blocks(N, 32), (unsigned)nsplit), 256, 0, s>>>(M, N, dZ, ld, part);
-  cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? launch_reduce_splits(N, nsplit, part, N, db, s) : e;
+cudaError_t launch_bias_grad(int64_t M, const BiasSegs &sg, int nsplit, cudaStream_t s) {
+  unsigned nx = 0;
+  for (int l = 0; l < kBiasSegs; ++l) nx += blocks(sg.N[l], 32);
+  k_bias_grad<<<dim3(nx, (unsigned)nsplit), 256, 0, s>>>(M, sg);
+  return cudaGetLastError();
 }
 cudaError_t launch_adam(int64_t n, float *w, const float *g, float *m, float *v, float lr, float b1,
                         float b2, float eps, int step, __nv_bfloat16 *w_bf, __nv_bfloat16 *wT_bf,
@@ -171,21 +180,15 @@ cudaError_t launch_adam(int64_t n, float *w, const float *g, float *m, float *v,
   k_adam<<<blocks(n, 256), 256, 0, s>>>(n, w, g, m, v, lr, b1, b2, eps, bc1, bc2, w_bf, wT_bf, rows, cols);
   return cudaGetLastError();
 }
-cudaError_t launch_adam_sched_all(int64_t n, float *w, const float *g, float *m, float *v, const float *sched,
+cudaError_t launch_adam_sched_all(int64_t n, float *w, float *m, float *v, const float *sched,
                                   const int64_t *step, float b1, float b2, float eps, const AdamSegs &segs,
                                   cudaStream_t s) {
-  k_adam_sched_all<<<blocks(n, 256), 256, 0, s>>>(n, w, g, m, v, sched, step, b1, b2, eps, segs);
+  k_adam_sched_all<<<blocks(n, 256), 256, 0, s>>>(n, w, m, v, sched, step, b1, b2, eps, segs);
   return cudaGetLastError();
 }
-cudaError_t launch_gather_rows_step(int64_t nrows, int ncol, const int32_t *idx, const int64_t *step,
-                                    int64_t nbatch, const float *in, int ldin, float *out, int ldout,
-                                    cudaStream_t s) {
-  k_gather_rows_step<<<blocks(nrows * ncol, 256), 256, 0, s>>>(nrows, ncol, idx, step, nbatch, in, ldin, out,
-                                                               ldout);
-  return cudaGetLastError();
-}
-cudaError_t launch_step_inc(int64_t *step, cudaStream_t s) {
-  k_step_inc<<<1, 32, 0, s>>>(step);
+cudaError_t launch_gather_batch(int64_t nrows, int ncol, const int32_t *idx, const int64_t *step, int64_t nbatch,
+                                const float *X, const float *T, __nv_bfloat16 *Xb, float *Tb, cudaStream_t s) {
+  k_gather_batch<<<blocks(nrows * ncol, 256), 256, 0, s>>>(nrows, ncol, idx, step, nbatch, X, T, Xb, Tb);
   return cudaGetLastError();
 }
 cudaError_t launch_to_bf16(int64_t n, const float *in, __nv_bfloat16 *out, cudaStream_t s) {

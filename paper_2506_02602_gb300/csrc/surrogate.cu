@@ -225,29 +225,53 @@ constexpr int kGradSplit = 16;
 constexpr int kGraphSteps = 8;
 
 struct TrainBufs {
-  float *Xb = nullptr, *Tb = nullptr, *Y = nullptr, *loss = nullptr, *part = nullptr;
+  float *Xb = nullptr, *Tb = nullptr, *Y = nullptr, *loss = nullptr;
   float *Z[3] = {}, *dH = nullptr;
-  __nv_bfloat16 *Xbf = nullptr, *H[3] = {}, *dY = nullptr, *dZ = nullptr;
+  // the split gradients' partial sums, per layer: every layer's are alive until the update
+  float *part[kSurLayers] = {}, *part_b[kSurLayers] = {};
+  // dZ per layer: a layer's is read by its weight gradient while the next one's is written
+  __nv_bfloat16 *Xbf = nullptr, *H[3] = {}, *dY = nullptr, *dZ[3] = {};
   void release() {
-    cudaFree(Xb); cudaFree(Tb); cudaFree(Y); cudaFree(loss); cudaFree(part); cudaFree(dH); cudaFree(Xbf);
-    cudaFree(dY); cudaFree(dZ);
-    for (int i = 0; i < 3; ++i) { cudaFree(Z[i]); cudaFree(H[i]); }
+    cudaFree(Xb); cudaFree(Tb); cudaFree(Y); cudaFree(loss); cudaFree(dH); cudaFree(Xbf);
+    cudaFree(dY);
+    for (int i = 0; i < 3; ++i) { cudaFree(Z[i]); cudaFree(H[i]); cudaFree(dZ[i]); }
+    for (int l = 0; l < kSurLayers; ++l) { cudaFree(part[l]); cudaFree(part_b[l]); }
   }
   cudaError_t alloc(int64_t B) {
     SCHK(cudaMalloc(&Xb, B * kSurIn * sizeof(float)));
     SCHK(cudaMalloc(&Tb, B * kSurOut * sizeof(float)));
     SCHK(cudaMalloc(&Y, B * kSurOut * sizeof(float)));
     SCHK(cudaMalloc(&loss, sizeof(float)));
-    SCHK(cudaMalloc(&part, (size_t)kGradSplit * kSurHidden * kSurHidden * sizeof(float)));
+    for (int l = 0; l < kSurLayers; ++l) {
+      SCHK(cudaMalloc(&part[l], (size_t)kGradSplit * kSurN[l] * kSurK[l] * sizeof(float)));
+      SCHK(cudaMalloc(&part_b[l], (size_t)kGradSplit * kSurN[l] * sizeof(float)));
+    }
     SCHK(cudaMalloc(&dH, B * kSurHidden * sizeof(float)));
     SCHK(cudaMalloc(&Xbf, B * kSurIn * sizeof(__nv_bfloat16)));
     SCHK(cudaMalloc(&dY, B * kSurOut * sizeof(__nv_bfloat16)));
-    SCHK(cudaMalloc(&dZ, B * kSurHidden * sizeof(__nv_bfloat16)));
     for (int i = 0; i < 3; ++i) {
+      SCHK(cudaMalloc(&dZ[i], B * kSurHidden * sizeof(__nv_bfloat16)));
       SCHK(cudaMalloc(&Z[i], B * kSurHidden * sizeof(float)));
       SCHK(cudaMalloc(&H[i], B * kSurHidden * sizeof(__nv_bfloat16)));
     }
     return cudaSuccess;
+  }
+};
+
+// A second stream for the weight gradients, which nothing needs before the update: they run
+// beside the chain of input gradients.  ev[l] marks layer l's output gradient, ev[kSurLayers] the end.
+struct SideStream {
+  cudaStream_t st = nullptr;
+  cudaEvent_t ev[kSurLayers + 1] = {};
+  cudaError_t create() {
+    SCHK(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+    for (cudaEvent_t &x : ev) SCHK(cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
+    return cudaSuccess;
+  }
+  void release() {
+    for (cudaEvent_t x : ev)
+      if (x) cudaEventDestroy(x);
+    if (st) cudaStreamDestroy(st);
   }
 };
 
@@ -263,17 +287,17 @@ static cudaError_t trace_copy(void *dst, const void *src, size_t bytes, cudaStre
   return dst ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToDevice, st) : cudaSuccess;
 }
 
-// Forward with saved activations, MSE over the 9 outputs, backward into s->grad.
-// X: normalised features [B x 16] (fp32, also converted to bf16), T: normalised targets.
-// tr (nullable) receives copies of the intermediates.
-static cudaError_t forward_backward(Surrogate *s, TrainBufs &b, int64_t B, cudaStream_t st,
-                                    const Trace *tr = nullptr) {
-  SCHK(launch_to_bf16(B * kSurIn, b.Xb, b.Xbf, st));
+// Forward with saved activations, MSE over the 9 outputs, backward into the partial sums of
+// b.part and b.part_b.  b.Xbf: normalised features [B x 16] (bf16), b.Tb: normalised targets.
+// step (nullable): a captured step's counter, advanced by the loss kernel.  side (nullable): the
+// weight gradients' stream.  tr (nullable) receives copies of the intermediates.
+static cudaError_t forward_backward(Surrogate *s, TrainBufs &b, int64_t B, cudaStream_t st, int64_t *step = nullptr,
+                                    SideStream *side = nullptr, const Trace *tr = nullptr) {
   SCHK(layer_forward(s, 0, B, b.Xbf, b.Z[0], b.H[0], nullptr, st));
   SCHK(layer_forward(s, 1, B, b.H[0], b.Z[1], b.H[1], nullptr, st));
   SCHK(layer_forward(s, 2, B, b.H[1], b.Z[2], b.H[2], nullptr, st));
   SCHK(layer_forward(s, 3, B, b.H[2], nullptr, nullptr, b.Y, st));
-  SCHK(launch_mse(B, NSP, kSurOut, b.Y, b.Tb, kSurOut, b.dY, kSurOut, b.loss, st));
+  SCHK(launch_mse(B, NSP, kSurOut, b.Y, b.Tb, kSurOut, b.dY, kSurOut, b.loss, step, st));
   const size_t slab = (size_t)B * kSurHidden;
   if (tr) {
     for (int l = 0; l < 3; ++l) {
@@ -284,42 +308,66 @@ static cudaError_t forward_backward(Surrogate *s, TrainBufs &b, int64_t B, cudaS
   }
   // layer l: input Hin [B x K], output gradient G [B x N] (bf16)
   const __nv_bfloat16 *Hin[kSurLayers] = {b.Xbf, b.H[0], b.H[1], b.H[2]};
-  const __nv_bfloat16 *G = b.dY;
+  const __nv_bfloat16 *G[kSurLayers] = {b.dZ[0], b.dZ[1], b.dZ[2], b.dY};
+  const cudaStream_t sw = side ? side->st : st;
   for (int l = kSurLayers - 1; l >= 0; --l) {
     const int N = kSurN[l], K = kSurK[l];
+    if (side) {
+      SCHK(cudaEventRecord(side->ev[l], st));
+      SCHK(cudaStreamWaitEvent(sw, side->ev[l], 0));
+    }
     // dW[n, k] = sum_m G[m, n] Hin[m, k]
     // (split-K over the batch into b.part, then a fixed-order reduction)
     GemmArgs gw{};
     gw.M = N; gw.N = K; gw.K = B;
-    gw.A = G; gw.sam = 1; gw.sak = N;
+    gw.A = G[l]; gw.sam = 1; gw.sak = N;
     gw.B = Hin[l]; gw.sbn = 1; gw.sbk = K;
     gw.alpha = 1.0f;
-    gw.Cf = b.part; gw.ldc = K;
+    gw.Cf = b.part[l]; gw.ldc = K;
     gw.split = kGradSplit;
     gw.split_ld = (int64_t)N * K;
     gw.err = s->tc_err;
-    SCHK(launch_gemm(gw, st));
-    SCHK(launch_reduce_splits((int64_t)N * K, kGradSplit, b.part, (int64_t)N * K, s->grad + s->off_W[l], st));
-    SCHK(launch_bias_grad(B, N, G, N, b.part, kGradSplit, s->grad + s->off_b[l], st));
+    SCHK(launch_gemm(gw, sw));
     if (l == 0) break;
     // dHin[m, k] = sum_n G[m, n] W[n, k] (W^T stored [K x N])
     // and in the same epilogue G for layer l-1: dZ = dHin * GELU'(Z_{l-1}) (bf16); the fp32
     // dHin itself is stored only for a trace
     GemmArgs gx{};
     gx.M = B; gx.N = K; gx.K = N;
-    gx.A = G; gx.sam = N; gx.sak = 1;
+    gx.A = G[l]; gx.sam = N; gx.sak = 1;
     gx.B = s->WT[l]; gx.sbn = N; gx.sbk = 1;
     gx.alpha = 1.0f;
     gx.Cf = (tr && tr->dH) ? b.dH : nullptr; gx.ldc = K;
-    gx.Cb = b.dZ; gx.ldcb = K;
+    gx.Cb = b.dZ[l - 1]; gx.ldcb = K;
     gx.dgelu_z = b.Z[l - 1]; gx.ldz = K;
     gx.err = s->tc_err;
     SCHK(launch_gemm(gx, st));
     if (tr) {
       SCHK(trace_copy(tr->dH ? tr->dH + (l - 1) * slab : nullptr, b.dH, slab * sizeof(float), st));
-      SCHK(trace_copy(tr->G ? tr->G + (l - 1) * slab : nullptr, b.dZ, slab * sizeof(__nv_bfloat16), st));
+      SCHK(trace_copy(tr->G ? tr->G + (l - 1) * slab : nullptr, b.dZ[l - 1], slab * sizeof(__nv_bfloat16), st));
     }
-    G = b.dZ;
+  }
+  BiasSegs bs{};
+  static_assert(kBiasSegs == kSurLayers, "one bias per layer");
+  for (int l = 0; l < kSurLayers; ++l) {
+    bs.dZ[l] = G[l];
+    bs.part[l] = b.part_b[l];
+    bs.N[l] = kSurN[l];
+  }
+  SCHK(launch_bias_grad(B, bs, kGradSplit, st));
+  if (side) {
+    SCHK(cudaEventRecord(side->ev[kSurLayers], sw));
+    SCHK(cudaStreamWaitEvent(st, side->ev[kSurLayers], 0));
+  }
+  return cudaSuccess;
+}
+
+// The gradient from forward_backward's partial sums into s->grad.
+static cudaError_t reduce_grad(Surrogate *s, const TrainBufs &b, cudaStream_t st) {
+  for (int l = 0; l < kSurLayers; ++l) {
+    const int64_t nw = (int64_t)kSurN[l] * kSurK[l];
+    SCHK(launch_reduce_splits(nw, kGradSplit, b.part[l], nw, s->grad + s->off_W[l], st));
+    SCHK(launch_reduce_splits(kSurN[l], kGradSplit, b.part_b[l], kSurN[l], s->grad + s->off_b[l], st));
   }
   return cudaSuccess;
 }
@@ -482,7 +530,9 @@ static int surrogate_pass(chem_ctx *ctx, const float *d_X, const float *d_T, int
   if (e == cudaSuccess) e = cudaMemcpyAsync(b.Xb, d_X, B * kSurIn * sizeof(float), cudaMemcpyDeviceToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b.Tb, d_T, B * kSurOut * sizeof(float), cudaMemcpyDeviceToDevice, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(b.loss, 0, sizeof(float), st);
-  if (e == cudaSuccess) e = forward_backward(s, b, B, st, tr);
+  if (e == cudaSuccess) e = launch_to_bf16(B * kSurIn, b.Xb, b.Xbf, st);
+  if (e == cudaSuccess) e = forward_backward(s, b, B, st, nullptr, nullptr, tr);
+  if (e == cudaSuccess) e = reduce_grad(s, b, st);
   if (e == cudaSuccess && d_Y) e = cudaMemcpyAsync(d_Y, b.Y, B * kSurOut * sizeof(float), cudaMemcpyDeviceToDevice, st);
   if (e == cudaSuccess && h_grad)
     e = cudaMemcpyAsync(h_grad, s->grad, (size_t)kSurParams * sizeof(float), cudaMemcpyDeviceToHost, st);
@@ -686,6 +736,7 @@ int chem_surrogate_train(chem_ctx *ctx, const chem_pairs *pairs, int64_t npairs,
   cudaGraph_t graph[4] = {nullptr, nullptr, nullptr, nullptr};
   cudaGraphExec_t exec[4] = {nullptr, nullptr, nullptr, nullptr};
   cudaEvent_t up_done[2] = {nullptr, nullptr};
+  SideStream side;
   auto release_graph = [&]() {
     for (int i = 0; i < 4; ++i) {
       if (exec[i]) cudaGraphExecDestroy(exec[i]);
@@ -693,6 +744,7 @@ int chem_surrogate_train(chem_ctx *ctx, const chem_pairs *pairs, int64_t npairs,
     }
     for (int i = 0; i < 2; ++i)
       if (up_done[i]) cudaEventDestroy(up_done[i]);
+    side.release();
     if (ps) cudaStreamDestroy(ps);
     cudaFree(dsched);
     cudaFree(dstep);
@@ -709,11 +761,14 @@ int chem_surrogate_train(chem_ctx *ctx, const chem_pairs *pairs, int64_t npairs,
   if (e == cudaSuccess) e = cudaMemset(dstep, 0, sizeof(int64_t));
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ps, cudaStreamNonBlocking);
   for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&up_done[i], cudaEventDisableTiming);
+  if (e == cudaSuccess) e = side.create();
   if (e == cudaSuccess) e = gemm_prepare();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // features and statistics are done
   int32_t *idxs[2] = {idx, idx2};
   static_assert(kAdamSegs == 2 * kSurLayers, "one weight and one bias segment per layer");
   AdamSegs sg{};  // Adam on every parameter in one launch (the layout W0 b0 W1 b1 ...)
+  sg.nsplit = kGradSplit;
+  static_assert(kSurIn == kSurOut, "a batch's features and targets are gathered together");
   for (int l = 0; l < kSurLayers; ++l) {
     sg.end[2 * l] = s->off_b[l];
     sg.end[2 * l + 1] = s->off_b[l] + kSurN[l];
@@ -721,17 +776,16 @@ int chem_surrogate_train(chem_ctx *ctx, const chem_pairs *pairs, int64_t npairs,
     sg.wT_bf[2 * l] = s->WT[l];
     sg.rows[2 * l] = kSurN[l];
     sg.cols[2 * l] = kSurK[l];
+    sg.part[2 * l] = b.part[l];
+    sg.part[2 * l + 1] = b.part_b[l];
     sg.rows[2 * l + 1] = 1;
     sg.cols[2 * l + 1] = kSurN[l];
   }
   auto capture_step = [&](int gi) {
-    cudaError_t ce = launch_gather_rows_step(B, kSurIn, idxs[gi], dstep, nb, X, kSurIn, b.Xb, kSurIn, ps);
-    if (ce == cudaSuccess) ce = launch_gather_rows_step(B, kSurOut, idxs[gi], dstep, nb, Tg, kSurOut, b.Tb, kSurOut, ps);
-    if (ce == cudaSuccess) ce = forward_backward(s, b, B, ps);
+    cudaError_t ce = launch_gather_batch(B, kSurIn, idxs[gi], dstep, nb, X, Tg, b.Xbf, b.Tb, ps);
+    if (ce == cudaSuccess) ce = forward_backward(s, b, B, ps, dstep, &side);
     if (ce == cudaSuccess)
-      ce = launch_adam_sched_all(kSurParams, s->param, s->grad, s->m, s->v, dsched, dstep, 0.9f, 0.999f, 1e-8f, sg,
-                                 ps);
-    if (ce == cudaSuccess) ce = launch_step_inc(dstep, ps);
+      ce = launch_adam_sched_all(kSurParams, s->param, s->m, s->v, dsched, dstep, 0.9f, 0.999f, 1e-8f, sg, ps);
     return ce;
   };
   // graph g = gi (one step) and g = 2 + gi (kGraphSteps steps) for permutation buffer gi:
