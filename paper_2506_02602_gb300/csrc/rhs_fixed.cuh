@@ -58,12 +58,20 @@ __shared__ int4 s_qe[2][NSP][3];
 __shared__ int4 s_qg[2][NSP][4];
 
 __device__ __forceinline__ int4 pack_q(const QCoef &a, const QCoef &b) { return make_int4(a.h, a.l, b.h, b.l); }
-__device__ __forceinline__ void load_fixed_tables(const MechTables &mt) {
-  load_exp2_tables();
-  load_log2_table();
+// solve_T_fixed's table
+__device__ __forceinline__ void load_energy_table(const MechTables &mt) {
   for (int i = threadIdx.x; i < 2 * NSP; i += blockDim.x) {
     const int r = i / NSP, k = i % NSP;
     for (int j = 0; j < 3; ++j) s_qe[r][k][j] = pack_q(mt.qe[r][k][2 * j], mt.qe[r][k][2 * j + 1]);
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ void load_fixed_tables(const MechTables &mt) {
+  load_exp2_tables();
+  load_log2_table();
+  load_energy_table(mt);
+  for (int i = threadIdx.x; i < 2 * NSP; i += blockDim.x) {
+    const int r = i / NSP, k = i % NSP;
     s_qg[r][k][0] = pack_q(mt.qg[r][k][0], mt.qg[r][k][1]);
     s_qg[r][k][1] = pack_q(mt.qgt[r][k][0], mt.qgt[r][k][1]);
     s_qg[r][k][2] = pack_q(mt.qgt[r][k][2], mt.qgt[r][k][3]);

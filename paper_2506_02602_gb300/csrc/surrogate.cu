@@ -387,6 +387,22 @@ static cudaError_t adam_all(Surrogate *s, float lr, cudaStream_t st) {
   return cudaSuccess;
 }
 
+// The element matrix and the lists of its nonzero entries.
+static void set_elements(SurrogateConsts &c, const MechTables &mt) {
+  int pr = 0;
+  for (int el = 0; el < 3; ++el) {
+    for (int k = 0; k < NSP; ++k) {
+      c.E[el][k] = mt.Emat[el][k];
+      if (mt.Emat[el][k] == 0.0) continue;
+      c.el_k[el][c.el_n[el]++] = (int8_t)k;
+      c.sp_e[k][c.sp_n[k]++] = (int8_t)el;
+    }
+    for (int b = el; b < 3; ++b, ++pr)
+      for (int k = 0; k < NSP; ++k)
+        if (mt.Emat[el][k] != 0.0 && mt.Emat[b][k] != 0.0) c.pr_k[pr][c.pr_n[pr]++] = (int8_t)k;
+  }
+}
+
 static SurrogateConsts make_consts(const Surrogate *s, const chem_surrogate_gate &g,
                                    const MechTables &mt) {
   SurrogateConsts c{};
@@ -406,13 +422,7 @@ static SurrogateConsts make_consts(const Surrogate *s, const chem_surrogate_gate
   c.rate_max = g.rate_max;
   c.lam = s->lam;
   c.dt_power = s->dt_power;
-  for (int el = 0; el < 3; ++el) {
-    c.emask[el] = 0;
-    for (int k = 0; k < NSP; ++k) {
-      c.E[el][k] = mt.Emat[el][k];
-      c.emask[el] |= (mt.Emat[el][k] != 0.0) << k;
-    }
-  }
+  set_elements(c, mt);
   return c;
 }
 
@@ -579,11 +589,7 @@ int chem_surrogate_project(chem_ctx *ctx, int64_t n, const double *d_Y0, const d
   if (ldY < n) return sur_fail(ctx, CHEM_ERR_INVALID, "ldY < n");
   const MechTables &mt = chem_ctx_tables(ctx);
   SurrogateConsts c{};
-  for (int el = 0; el < 3; ++el)
-    for (int k = 0; k < NSP; ++k) {
-      c.E[el][k] = mt.Emat[el][k];
-      c.emask[el] |= (mt.Emat[el][k] != 0.0) << k;
-    }
+  set_elements(c, mt);
   const cudaError_t e = launch_project_check(c, n, d_Y0, d_Yp, ldY, d_Yout, (cudaStream_t)stream);
   return e == cudaSuccess ? CHEM_OK : sur_cuda(ctx, e, "projection");
 }

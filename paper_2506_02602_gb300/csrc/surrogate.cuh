@@ -52,7 +52,9 @@ struct SurrogateConsts {
   double lam;                           // Box-Cox lambda
   double dt_power;                      // targets scaled by (kSurDtRef / dt)^dt_power
   double E[3][NSP];                     // element mass fraction per unit species mass fraction
-  int32_t emask[3];                     // bit k set where E[el][k] != 0 (the sums skip the rest)
+  int8_t el_n[3], el_k[3][NSP];          // the species with E[el][k] != 0 (the sums skip the rest)
+  int8_t pr_n[6], pr_k[6][NSP];          // the same for the pairs of elements 00, 01, 02, 11, 12, 22
+  int8_t sp_n[NSP], sp_e[NSP][3];        // the elements of a species
 };
 
 cudaError_t launch_features(const MechTables &mt, int64_t n, const double *rho, const double *e,
@@ -84,7 +86,7 @@ cudaError_t launch_pack_weights(const __nv_bfloat16 *const (&W)[kSurLayers], uns
 size_t packed_weight_bytes();
 cudaError_t launch_mlp_tc(int64_t n, const float *X, const float *norm, const unsigned char *Wpk,
                           const float *const (&b)[kSurLayers], float *O, int *err, cudaStream_t s);
-// The fp64 element projection of the inference epilogue alone (only sc.E and sc.emask are
+// The fp64 element projection of the inference epilogue alone (only sc.E and its lists are
 // read): Yout = projection of Yp onto the element mass fractions of Y0 (planes, stride ld).
 cudaError_t launch_project_check(const SurrogateConsts &sc, int64_t n, const double *Y0,
                                  const double *Yp, int64_t ld, double *Yout, cudaStream_t s);

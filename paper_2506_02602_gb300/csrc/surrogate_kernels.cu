@@ -179,14 +179,15 @@ __global__ void k_normalize(int64_t n, int ncol, int ld, float *A, const float *
 // (cell_rhs_f32), whatever the context's variant: an estimate compared with a tolerance
 // of ~5e-4 T needs nothing finer; y1 - y0 is formed in fp64 first, so the defect does not
 // lose it to rounding.
-__device__ __forceinline__ bool posterior_error(const MechTables &mt, const double (&y0)[NSP],
-                                             const double (&y1)[NSP], float rho_f, float eR,
+template <int ST>
+__device__ __forceinline__ bool posterior_error(const MechTables &mt, const double *y0,
+                                             const double *y1, float rho_f, float eR,
                                              float T0, float T1f, float dtf, float &dT, float &rate) {
   float u0[NSP], u1[NSP], F0[NSP], F1[NSP];
 #pragma unroll
   for (int k = 0; k < NSP; ++k) {
-    u0[k] = d2f(y0[k]);
-    u1[k] = d2f(y1[k]);
+    u0[k] = d2f(y0[k * ST]);
+    u1[k] = d2f(y1[k * ST]);
   }
   const float invRho_f = __fdividef(1.0f, rho_f);
   float Ta = T0, Tb = T1f;
@@ -213,7 +214,7 @@ __device__ __forceinline__ bool posterior_error(const MechTables &mt, const doub
     const float *c = mt.f.ec[range][k];
     const float ukR =
         fmaf(T1f, fmaf(T1f, fmaf(T1f, fmaf(T1f, fmaf(T1f, c[4], c[3]), c[2]), c[1]), c[0]), c[5]) * mt.f.invW[k];
-    const float defect = d2f(y1[k] - y0[k]) - sdt * (F0[k] + 4.0f * Fm[k] + F1[k]);
+    const float defect = d2f(y1[k * ST] - y0[k * ST]) - sdt * (F0[k] + 4.0f * Fm[k] + F1[k]);
     sum = fmaf(fabsf(ukR - eR), fabsf(defect), sum);
     r = fmaxf(r, fmaxf(__fdividef(fabsf(F0[k]), fabsf(u0[k]) + 1e-6f), __fdividef(fabsf(F1[k]), fabsf(u1[k]) + 1e-6f)));
   }
@@ -228,21 +229,25 @@ __device__ __forceinline__ bool posterior_error(const MechTables &mt, const doub
 // appends rejected ones to the fallback list.
 // Weighted least-squares projection of the prediction y1 onto the element (H, O, N) mass
 // fractions of y0: Y'' = Y' - W E^T (E W E^T)^-1 r with W = diag(max(Y'_k, 1e-12)) and
-// r = E (Y' - Y0), in fp64 (terms with a zero element fraction skipped: uniform branches
-// on the masks).  rn and zn receive |r|^2 and |E Y0|^2 of the raw prediction (the
+// r = E (Y' - Y0), in fp64.  y0 and y1 are per-thread columns of shared memory, ST threads apart,
+// and the sums run over lists of the terms with a nonzero element fraction: under masks in
+// unrolled code the compiler computed all 189 products and selected 73 of them.
+// rn and zn receive |r|^2 and |E Y0|^2 of the raw prediction (the
 // residual gate's inputs).  Returns false, with y1 unchanged, when the 3x3 system is
 // singular or not finite.
-__device__ __forceinline__ bool project_elements(const SurrogateConsts &sc, const double (&y0)[NSP],
-                                                 double (&y1)[NSP], double &rn, double &zn) {
+template <int ST>
+__device__ __forceinline__ bool project_elements(const SurrogateConsts &sc, const double *y0, double *y1, double &rn,
+                                                 double &zn) {
   double z0[3] = {0.0, 0.0, 0.0}, r[3] = {0.0, 0.0, 0.0};
 #pragma unroll
   for (int el = 0; el < 3; ++el)
-#pragma unroll
-    for (int k = 0; k < NSP; ++k)
-      if ((sc.emask[el] >> k) & 1) {
-        z0[el] = fma(sc.E[el][k], y0[k], z0[el]);
-        r[el] = fma(sc.E[el][k], y1[k] - y0[k], r[el]);
-      }
+#pragma unroll 1
+    for (int i = 0; i < sc.el_n[el]; ++i) {
+      const int k = sc.el_k[el][i];
+      const double E = sc.E[el][k], a = y0[k * ST];
+      z0[el] = fma(E, a, z0[el]);
+      r[el] = fma(E, y1[k * ST] - a, r[el]);
+    }
   rn = 0.0;
   zn = 0.0;
 #pragma unroll
@@ -250,17 +255,18 @@ __device__ __forceinline__ bool project_elements(const SurrogateConsts &sc, cons
     rn = fma(r[el], r[el], rn);
     zn = fma(z0[el], z0[el], zn);
   }
-  double w[NSP], M[3][3];
-#pragma unroll
-  for (int k = 0; k < NSP; ++k) w[k] = max_pos(y1[k], 1e-12);
+  double M[3][3];
+  int pr = 0;
 #pragma unroll
   for (int a = 0; a < 3; ++a)
 #pragma unroll
-    for (int b = a; b < 3; ++b) {
+    for (int b = a; b < 3; ++b, ++pr) {
       double s = 0.0;
-#pragma unroll
-      for (int k = 0; k < NSP; ++k)
-        if (((sc.emask[a] & sc.emask[b]) >> k) & 1) s = fma(sc.E[a][k] * w[k], sc.E[b][k], s);
+#pragma unroll 1
+      for (int i = 0; i < sc.pr_n[pr]; ++i) {
+        const int k = sc.pr_k[pr][i];
+        s = fma(sc.E[a][k] * max_pos(y1[k * ST], 1e-12), sc.E[b][k], s);
+      }
       M[a][b] = s;
       M[b][a] = s;
     }
@@ -277,37 +283,51 @@ __device__ __forceinline__ bool project_elements(const SurrogateConsts &sc, cons
              M[0][2] * (M[1][0] * r[2] - r[1] * M[2][0])) * id;
   lamv[2] = (M[0][0] * (M[1][1] * r[2] - r[1] * M[2][1]) - M[0][1] * (M[1][0] * r[2] - r[1] * M[2][0]) +
              r[0] * (M[1][0] * M[2][1] - M[1][1] * M[2][0])) * id;
-#pragma unroll
+#pragma unroll 1
   for (int k = 0; k < NSP; ++k) {
     double corr = 0.0;
-#pragma unroll
-    for (int el = 0; el < 3; ++el)
-      if ((sc.emask[el] >> k) & 1) corr = fma(sc.E[el][k], lamv[el], corr);
-    y1[k] = fma(-w[k], corr, y1[k]);
+#pragma unroll 1
+    for (int i = 0; i < sc.sp_n[k]; ++i) {
+      const int el = sc.sp_e[k][i];
+      corr = fma(sc.E[el][k], el == 0 ? lamv[0] : el == 1 ? lamv[1] : lamv[2], corr);
+    }
+    const double y = y1[k * ST];
+    y1[k * ST] = fma(-max_pos(y, 1e-12), corr, y);
   }
   return true;
 }
 
 // The projection alone on given predictions (a check entry; see project_elements).
-__global__ void k_project_check(const __grid_constant__ SurrogateConsts sc, int64_t n,
-                                const double *__restrict__ Y0, const double *__restrict__ Yp,
-                                int64_t ld, double *__restrict__ Yout) {
+__global__ void __launch_bounds__(128)
+    k_project_check(const __grid_constant__ SurrogateConsts sc, int64_t n, const double *__restrict__ Y0,
+                    const double *__restrict__ Yp, int64_t ld, double *__restrict__ Yout) {
+  __shared__ double s_y[2 * NSP * 128];
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  double y0[NSP], y1[NSP];
+  double *y0 = s_y + threadIdx.x, *y1 = y0 + NSP * 128;
 #pragma unroll
   for (int k = 0; k < NSP; ++k) {
-    y0[k] = Y0[k * ld + i];
-    y1[k] = Yp[k * ld + i];
+    y0[k * 128] = Y0[k * ld + i];
+    y1[k * 128] = Yp[k * ld + i];
   }
   double rn, zn;
-  project_elements(sc, y0, y1, rn, zn);
+  project_elements<128>(sc, y0, y1, rn, zn);
 #pragma unroll
-  for (int k = 0; k < NSP; ++k) Yout[k * ld + i] = y1[k];
+  for (int k = 0; k < NSP; ++k) Yout[k * ld + i] = y1[k * 128];
 }
 
-// 4 blocks of 128 per SM (16 warps): the register cap of 128 costs 4 bytes of spill
-// stores, against 8 warps at the uncapped 255 registers.  The error test is inlined: as a
+// solve_T on a column, for what solve_T_fixed leaves.
+template <int ST>
+static __device__ __noinline__ bool solve_T_column(const MechTables &mt, const double *U, double eR, double *T) {
+  double Y[NSP];
+#pragma unroll
+  for (int k = 0; k < NSP; ++k) Y[k] = U[k * ST];
+  return solve_T(mt, Y, eR, *T);
+}
+
+// Bound by its FP64 instructions.  With the sums over lists and the temperature in fixed point a
+// call on 2M cells takes 4.0 instead of 4.6 ms (this kernel was 1.8 ms of them).
+// 4 blocks of 128 per SM (16 warps) at 128 registers, with the cell's states in shared memory.  The error test is inlined: as a
 // called function it took its state arrays by reference through a ~580-byte local
 // stack frame, and the kernel ran 10-14 % slower.
 template <int V>
@@ -318,9 +338,12 @@ __global__ void __launch_bounds__(128, 4)
                        const double *__restrict__ rho, const double *__restrict__ e, double *Y,
                        int64_t ld, double *T, int32_t *status, int32_t *nsteps, uint8_t *mask,
                        int32_t *fb_idx, unsigned int *fb_count, int64_t base) {
-  load_math_tables();
+  constexpr int ST = 128;
+  __shared__ double s_y[2 * NSP * ST];
+  load_energy_table(mt);
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
+  double *const y0 = s_y + threadIdx.x, *const y1 = y0 + NSP * ST;
   const float *x = Xraw + i * kSurIn;
   const float *o = O + i * kSurOut;
   // reason of a rejection (the first gate that fails), reported in the fallback mask
@@ -333,39 +356,44 @@ __global__ void __launch_bounds__(128, 4)
     inbox &= x[c] >= sc.fmin[c] - w && x[c] <= sc.fmax[c] + w;
   }
   if (!reason && !inbox) reason = kFbRange;
-  double y0[NSP], y1[NSP];
   const float unscale =
       sc.dt_power == 0.0 ? 1.0f : powf(d2f(dt) * (float)(1.0 / kSurDtRef), d2f(sc.dt_power));
 #pragma unroll
   for (int k = 0; k < NSP; ++k) {
-    y0[k] = Y[k * ld + i];
+    const double y = Y[k * ld + i];
     const float d = fmaf(o[k], sc.tstd[k], sc.tmean[k]) * unscale;
-    y1[k] = boxcox_step(y0[k], x[3 + k], d, (float)sc.lam);
+    y0[k * ST] = y;
+    y1[k * ST] = boxcox_step(y, x[3 + k], d, (float)sc.lam);
   }
   double rn = 0.0, zn = 0.0;
-  const bool solved = project_elements(sc, y0, y1, rn, zn);
+  const bool solved = project_elements<ST>(sc, y0, y1, rn, zn);
   if (!reason && !(rn <= (double)sc.resid_max * sc.resid_max * zn)) reason = kFbResidual;
   if (!reason && !solved) reason = kFbResidual;
   // the negativity test on the fp32-rounded result (a NaN fails it)
   bool neg = false;
 #pragma unroll
-  for (int k = 0; k < NSP; ++k) neg |= !(d2f(y1[k]) >= -sc.neg_tol);
+  for (int k = 0; k < NSP; ++k) neg |= !(d2f(y1[k * ST]) >= -sc.neg_tol);
   if (!reason && neg) reason = kFbNegative;
-  // temperature of the projected state (fp64 Newton from the input temperature)
+  // temperature of the projected state (Newton from the input temperature)
   const double eR = e[i] * (1.0 / R_U);
   double T1 = f2d(x[0]);
-  const bool tok = solve_T(mt, y1, eR, T1);
+  bool tok = mt.fixed_ok && solve_T_fixed<ST>(mt, y1, eR, T1);
+  if (!tok) {
+    double Tc = T1;
+    tok = solve_T_column<ST>(mt, y1, eR, &Tc);
+    T1 = Tc;
+  }
   const float T1f = d2f(T1);
   if (!reason && !(tok && fabsf(T1f - x[0]) <= sc.max_dT)) reason = kFbTemperature;
   if (!reason && sc.err_tol > 0.0f) {
     float dT = 0.0f, rate = 0.0f;
-    const bool jok = posterior_error(mt, y0, y1, d2f(rho[i]), d2f(eR), x[0], T1f, d2f(dt), dT, rate);
+    const bool jok = posterior_error<ST>(mt, y0, y1, d2f(rho[i]), d2f(eR), x[0], T1f, d2f(dt), dT, rate);
     if (!jok || !(sc.rate_max < 0.0f || rate <= sc.rate_max)) reason = kFbReactive;
     else if (!(dT <= sc.err_tol * T1f * (1.0f - 0.5f * rate + rate * rate * (1.0f / 12.0f)))) reason = kFbError;
   }
   if (!reason) {
 #pragma unroll
-    for (int k = 0; k < NSP; ++k) Y[k * ld + i] = y1[k];
+    for (int k = 0; k < NSP; ++k) Y[k * ld + i] = y1[k * ST];
     T[i] = T1;
     if (status) status[i] = CHEM_CELL_OK;
     if (nsteps) nsteps[i] = 0;
@@ -487,7 +515,7 @@ cudaError_t launch_one_box(int64_t *box_off, double *box_dt, int32_t *box_nsub, 
 cudaError_t launch_project_check(const SurrogateConsts &sc, int64_t n, const double *Y0,
                                  const double *Yp, int64_t ld, double *Yout, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_project_check<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(sc, n, Y0, Yp, ld, Yout);
+  k_project_check<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(sc, n, Y0, Yp, ld, Yout);
   return cudaGetLastError();
 }
 
