@@ -254,9 +254,9 @@ typedef struct {
 
 /* Compiled shapes of the persistent kernel: (threads per CTA, minimum resident CTAs
  * per SM, hence a register cap of min(255, 65536 / (threads * CTAs))):
- * 0 = (128, 2) [default, no cap in effect], 1 = (128, 3), 2 = (128, 4), 3 = (64, 6),
- * 4 = (64, 8), 5 = (256, 2) for fp64; for the mixed variant 0 = (128, 4) [default], 2 = (128, 2)
- * and 4 = (64, 16) with 9 species, 0 = (128, 3), 2 = (128, 2) with 13, the others as for fp64.
+ * 0 = (128, 3) [default], 1 = (128, 2), 2 = (128, 4), 3 = (64, 6), 4 = (64, 8), 5 = (256, 2)
+ * for fp64; for the mixed variant 0 = (128, 4) [default; (128, 3) with 13 species],
+ * 1 = (128, 3), 2 = (128, 2) and 4 = (64, 16) ((64, 8) with 13 species), the others as for fp64.
  * All run the same algorithm; the compiler contracts
  * multiply-adds per compiled kernel, so results of different shapes agree to rounding
  * (to the integration tolerance in ill-conditioned cells), not bit for bit.  Shape 0

@@ -202,13 +202,14 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_lsrk_persistent(const __grid_co
   if (a.stats) accumulate_stats(a.stats, done_cells, tot_acc, tot_rej, tot_rhs, max_steps, hist);
 }
 
-// Threads per CTA and minimum resident CTAs per SM of each shape; shape 0 is the default.  The
-// mixed variant's shapes 0 and 2 are exchanged: its default keeps 16 warps per SM (12 with
-// 13 species; its per-thread columns allow no more), which runs the ragged AMR batch in 70 ms
-// against 90 for 128 x 2 (and 83 for the 64-register shape 4).
+// Threads per CTA and minimum resident CTAs per SM of each shape; shape 0 is the default.  fp64: 12
+// warps per SM run the 3.46 M-cell ragged AMR batch in 255 ms, 8 (128 x 2, which had no spills
+// when a cell's vectors were in registers) in 280, and the 128-register shapes in 259 to 297.
+// Mixed: its per-thread columns allow 16 warps (12 with 13 species), 59 ms against 65 at 12 and 80
+// at 8 (and 73 for the 64-register shape 4).
 static constexpr int kShapeBlock[CHEM_BATCH_SHAPES] = {128, 128, 128, 64, 64, 256};
 template <int V>
-constexpr int kShapeMinB[CHEM_BATCH_SHAPES] = {2, 3, 4, 6, 8, 2};
+constexpr int kShapeMinB[CHEM_BATCH_SHAPES] = {3, 2, 4, 6, 8, 2};
 template <>
 constexpr int kShapeMinB<CHEM_VARIANT_MIXED>[CHEM_BATCH_SHAPES] = {NSP <= 9 ? 4 : 3, 3, 2, 6, NSP <= 9 ? 16 : 8, 2};
 
