@@ -42,7 +42,7 @@ Legs of one run (rank 0 prints one JSON line):
   value     device-resident throughput (cells/s) of the headline variant;
   e2e       the same through chem_integrate_host: host buffers (pinned), H2D + D2H
             copies inside the timed region;
-  roofline  credited FP64 flops per launch / CUDA-event launch time vs the FP64 peak;
+  roofline  FP64-pipe flops per launch / CUDA-event launch time vs the FP64 peak;
   cpu_baseline  the CPU oracle on a bounded sample of the same workload (rank 0, N=1).
 --impl reference runs only the oracle (the deliberately slow plain CPU program).
 Under torchrun each rank integrates its own full slice (independent cells, weak
@@ -335,10 +335,8 @@ MLP_FLOPS_PER_ROW = 2 * (16 * 256 + 256 * 256 * 2 + 256 * 16)  # padded 16-256-2
 # DRAM bytes (read + write) per cell of one k_lsrk launch (dram__bytes_read.sum +
 # dram__bytes_write.sum), from an ncu capture of the 131,072-cell slice, scaled by the
 # cell count; to be set to None whenever the kernel changes until it is captured again.
-# fp64: 12.84 MB per 131,072-cell launch (mean of 4 launches of the current kernel);
-# mixed (32 warps per SM, spilling): 12.75 MB read + 7.75 MB written (spill lines evicted
-# from L2), mean of 4 launches of the current kernel
-TRAFFIC_PER_CELL = {"fp64": 12.841984e6 / 131072, "mixed": 20.507712e6 / 131072}
+# fp64: 12.95 MB read per 131,072-cell launch, mixed: 13.87 MB read + 0.26 MB written
+TRAFFIC_PER_CELL = {"fp64": 12.95e6 / 131072, "mixed": 14.13e6 / 131072}
 
 
 def _bf16_peak():
@@ -465,7 +463,7 @@ def mech13_leg(steps, dev, stream, flush, ref9):
             flops = roofline.launch_flops(steps_tot, n, m13)
         else:
             flops = roofline.launch_flops_mixed_fp64(steps_tot, n, m13)
-        achieved = flops / (ms * 1e-3) / 1e9
+        achieved = steps_tot * roofline.step_flops_fp64_pipe(m13, variant) / (ms * 1e-3) / 1e9
         res[variant] = {"ms": ms, "cells_per_s": n / (ms * 1e-3), "attempted_steps": steps_tot,
                         "credited_gflop_per_launch": flops / 1e9, "achieved_gflops": achieved,
                         "frac_of_fp64_peak": achieved / roofline.FP64_PEAK_GFLOPS}
@@ -1023,10 +1021,12 @@ def run_ours(args, rank, world, local):
         absY = float(np.max(np.abs(r["Y"] - ref["Y"])))
         if v == "fp64":
             flops = roofline.launch_flops(int(r["nsteps"].sum()), n, mech)
-            note = "fp64 pipe; credited flops (exp/log = 20) / CUDA-event launch time"
+            note = ("fp64 pipe; flops left on it (products of concentrations, registers, control; the rest of the "
+                    "right-hand side is 64-bit fixed point) / CUDA-event launch time; credited: the algorithm's")
         elif v == "mixed":
             flops = roofline.launch_flops_mixed_fp64(int(r["nsteps"].sum()), n, mech)
-            note = "fp64 pipe; credited fp64 part only (temperature solve, Gibbs, hi/lo splits for ln Kc, fp64 registers, control)"
+            note = ("fp64 pipe; flops left on it (registers, control; the right-hand side is fp32 and double-float: the "
+                    "kernel is bound by the latency of its fp32 chains); credited: the algorithm's fp64 part")
         if v == "hybrid":
             # the fused network kernel, timed alone on the surrogate leg's rows
             mk = sur["mlp_kernel"]
@@ -1035,11 +1035,13 @@ def run_ours(args, rank, world, local):
                   "note": "the network's tcgen05 BF16 kernel, timed alone on "
                           f"{mk['rows']} rows; peak = measured cuBLAS bf16 burst"}
         else:
-            achieved = flops / (r["kernel_ms"] * 1e-3) / 1e9
+            credited = flops / (r["kernel_ms"] * 1e-3) / 1e9
+            achieved = (int(r["nsteps"].sum()) * roofline.step_flops_fp64_pipe(mech, v)
+                        / (r["kernel_ms"] * 1e-3) / 1e9)
             tpc = TRAFFIC_PER_CELL.get(v)
             rl = {"bound": "alu", "achieved": achieved, "peak": roofline.FP64_PEAK_GFLOPS,
                   "unit": "GFLOP/s", "frac": achieved / roofline.FP64_PEAK_GFLOPS,
-                  "traffic": None if tpc is None else tpc * n, "note": note +
+                  "credited_gflops": credited, "traffic": None if tpc is None else tpc * n, "note": note +
                   "; traffic = ncu DRAM bytes per cell on a 131,072-cell slice x cells"}
         summary[v] = {
             "value": job_rate(world, n, args.steps, r["elapsed"]), "ms_per_step": 1e3 * r["elapsed"] / args.steps,

@@ -19,7 +19,7 @@
 // On GB300 an FP64 instruction costs a warp 64 cycles of its sub-partition whatever else the
 // warp does, a double-float multiply-add about 13 (6 with the packed f32x2 forms).  With the
 // temperature solve and the Gibbs functions in fp64 the FP64 pipe was 82 % busy and the issue
-// slots 26 %; now the pipe is about 40 % busy (the solution and error registers, the norm, the
+// slots 26 %; now the pipe is 51 % busy (the solution and error registers, the norm, the
 // evaluations in fp64) and issue 53 %.  What bounds the kernel is the latency of dependent
 // fp32 operations at 16 warps an SM, and it runs the 1M-cell detonation slice in 7.9 ms
 // instead of 16.1 (the 151,979-cell 13-species slice in 2.1 instead of 3.4).

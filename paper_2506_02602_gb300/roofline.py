@@ -15,8 +15,11 @@ side is counted from the mechanism structure in the formulation the kernels use:
 Add, multiply, compare-free min/max and divide count 1 flop, an FMA 2, and every
 exp / log / exp10 / log10 / sqrt is credited a fixed TRANSCENDENTAL flops.  The FP64
 pipe of GB300 spends about 20 FMA slots (40 flops) on a library exp, so this credit is
-conservative: the reported fraction understates the FP64 pipe's busy time, which the
-ncu summary reports separately.
+conservative.
+
+Most of that work has left the FP64 pipe (64-bit fixed point on the integer pipe, double-float
+on the FP32 pipe), so credited work per second can exceed the FP64 peak; the fraction of the
+peak is reported for what stays on the pipe (step_flops_fp64_pipe).
 """
 from __future__ import annotations
 
@@ -143,6 +146,44 @@ def step_flops_mixed_fp64(mech: dict | None = None, scheme: int = 0) -> int:
 def launch_flops_mixed_fp64(total_attempted_steps: int, ncells: int, mech: dict | None = None,
                             scheme: int = 0) -> float:
     return float(total_attempted_steps) * step_flops_mixed_fp64(mech, scheme) + float(ncells) * cell_flops(mech)
+
+
+def step_flops_fp64_pipe(mech: dict | None = None, variant: str = "fp64", scheme: int = 0) -> int:
+    """The flops of one attempted step that the kernels leave on the FP64 pipe, the unit the FP64
+    peak is of.  fp64: per right-hand side the concentrations and their total, 1/T (a cubic
+    reciprocal: 3 FMAs), per stoichiometry the products, the net rate and its updates, the
+    third-body sums over their lists, the fall-off algebra, and F_k; the temperature solve, Gibbs
+    functions, exponents, exponentials and logarithms are integer work.  mixed: nothing of a
+    right-hand side.  Both: the register updates, the WRMS norm and the control."""
+    nsp, rxs = _structure(mech)
+    s = STAGES[scheme]
+    if variant == "fp64":
+        rhs = 3 * nsp + 6
+        seen = set()
+        for j, (nr, npr, typ, _) in enumerate(rxs):
+            key = j if mech is None else (tuple(mech["nu_f"][j]), tuple(mech["nu_r"][j]))
+            if key not in seen:
+                rhs += (nr - 1) + (npr - 1) + 2 + 1 + nr + npr
+            else:
+                rhs += 1                       # k_f added to its stoichiometry's
+            seen.add(key)
+            if typ != 0:
+                eff = None if mech is None else mech["eff"][j]
+                rhs += 2 * (nsp if eff is None else min(int(sum(x != 1.0 for x in eff)), int(sum(x != 0.0 for x in eff))))
+            if typ == 1:
+                rhs += 1
+            if typ == 2:
+                rhs += 2 + 6 + 2 + 7 + 2 + 8 + 1 + 2 + 6 + 3  # k0 M / (k + k0 M), F_cent, x, d, F
+        if scheme == 0:
+            updates = s * (3 + nsp * 3 * 2)
+        else:
+            updates = nsp * 2 * (s * (s - 1) // 2 + 2 * s) + s
+    else:
+        rhs = 0
+        updates = s * (3 + nsp * 2 * 2)
+    wrms = nsp * (2 + (6 if variant == "fp64" else 4) + 1 + 2) + 1
+    control = 4 * T_SQRT + 3
+    return s * rhs + updates + wrms + control
 
 
 # FP64 peak of GB300 derived from unit counts and clocks: 152 SMs x 2 FP64 FMA lanes per
