@@ -237,6 +237,8 @@ int build_tables(const chem_mechanism *m, MechTables *t) {
     t->troe_q3[j] = t->troe_i3[j] * log2e;
     t->troe_q1[j] = t->troe_i1[j] * log2e;
     t->troe_q2[j] = t->troe_T2[j] * log2e;
+    // exp(-T** / T) stays below to_q52's limit
+    if (kRx[j].troe_n == 4 && !(t->troe_q2[j] > -128000.0)) t->fixed_ok = 0;
   }
   for (int r = 0; r < 2 && t->fixed_ok; ++r) {
     int S = 13;

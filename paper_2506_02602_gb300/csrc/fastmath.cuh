@@ -68,6 +68,11 @@ static __device__ __noinline__ double exp_t(double x) {
   return fma(ts, p, ts);
 }
 
+// x is a NaN, on the integer pipe
+__device__ __forceinline__ bool is_nan(double x) {
+  return (__double_as_longlong(x) & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL;
+}
+
 // x clamped to [-lim, lim] for lim > 0 (a NaN gives +-lim)
 __device__ __forceinline__ double clamp_abs(double x, double lim) {
   const long long b = __double_as_longlong(x);
@@ -127,7 +132,7 @@ __device__ __forceinline__ unsigned long long abs_q(double x) {
   return m >> min(62 - Q - e, 63);
 }
 
-// x in Q52, limited to +-1009.9 (a factor e^+-700)
+// x in Q52, limited to +-1009.9 (a factor e^+-700); a NaN gives a limit, so callers look for it
 __device__ __forceinline__ long long to_q52(double x) {
   const long long v = (long long)abs_q<52>(clamp_abs(x, 1009.875));
   return __double2hiint(x) < 0 ? -v : v;

@@ -228,7 +228,8 @@ __device__ __forceinline__ double rate_fixed(const MechTables &mt, const RateInp
       const double x = fma(-0.67, lFc, lPr - 0.4 * kLog2_10);
       const double d = fma(-0.14, x, fma(-1.27, lFc, 0.75 * kLog2_10));
       const double d2 = d * d;
-      const long long lF = to_q52(lFc * (d2 * rcp3(fma(x, x, d2))));
+      const double f2 = lFc * (d2 * rcp3(fma(x, x, d2)));
+      const long long lF = to_q52(f2);
       double F;
       if constexpr (kK && R.troe_n != 4) {
         const double2 w = exp2_q52(lF, lK);
@@ -237,7 +238,9 @@ __device__ __forceinline__ double rate_fixed(const MechTables &mt, const RateInp
       } else {
         F = exp2_q52(lF);
       }
-      kf = kf > 0.0 ? kf * F : 0.0;  // without third bodies F is not a number
+      // Without third bodies log Pr is infinite and the rate zero.  Else a factor that is no number
+      // (F_cent zero, negative or NaN) makes the rate none, as in the general form: to_q52 has none.
+      kf = k0M > 0.0 ? kf * (is_nan(f2) ? f2 : F) : 0.0;
     } else if constexpr (kK) {
       K = exp2_q52(lK);
     }
