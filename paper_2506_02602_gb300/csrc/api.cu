@@ -255,13 +255,16 @@ int build_tables(const chem_mechanism *m, MechTables *t) {
       }
       const double *g = t->gc[r][k];
       double gsum = 13.0 * std::fabs(g[0]) + std::fabs(g[5]) * log2e / 128.0 + std::fabs(g[0] + g[6]) * log2e;
-      double gt[4];
+      // the terms t .. t^4 add up in units of 2^-56: for 0 < t < 1 every partial sum lies between
+      // the negative terms' sum and the positive ones'
+      double gt[4], gpos = 0.0, gneg = 0.0;
       for (int i = 0; i < 4; ++i) {
         gt[i] = std::ldexp(-log2e * g[i + 1], S * (i + 1));
         gsum += std::fabs(gt[i]);
+        (gt[i] < 0.0 ? gneg : gpos) += std::fabs(gt[i]);
         if (!(std::fabs(gt[i]) < 64.0)) t->fixed_ok = 0;
       }
-      if (!(gsum < 1500.0) || !(std::fabs(g[0]) < 64.0)) t->fixed_ok = 0;
+      if (!(gpos < 127.0 && gneg < 127.0) || !(gsum < 1500.0) || !(std::fabs(g[0]) < 64.0)) t->fixed_ok = 0;
       if (!t->fixed_ok) break;
       t->qg[r][k][0] = qcoef(g[0], 56, 2);
       t->qg[r][k][1] = qcoef(-log2e * g[5], 44, 2);
