@@ -655,7 +655,7 @@ int chem_diag_fma_peak(int op, int32_t blocks, int32_t threads, int64_t iters, v
  * Diagnostic: the equilibrium exponents ln(1 / K_c,j) = sum_k nu_jk g_k / (R_u T)
  * + (sum_k nu_jk) ln(R_u T / p_ref) (Sec. 2.2.3: the reverse rates k_r = k_f / K_c of the
  * law of mass action) of every reaction of the context's mechanism at n temperatures
- * d_T (device, fp64, kelvin, > 0; non-positive values give NaN), written to d_out
+ * d_T (device, fp64, kelvin, > 0; values that are not positive and finite give NaN), written to d_out
  * (device, n * n_reactions fp64, row i = temperature i, the fp32 results widened
  * exactly), as the mixed-precision right-hand sides form them: form 0 the mixed
  * variant's (fp64 Gibbs functions summed as fp32 hi/lo pairs), form 1 the all-fp32 one of

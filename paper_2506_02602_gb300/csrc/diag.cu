@@ -97,6 +97,10 @@ __global__ void k_ln_inv_kc(const __grid_constant__ MechTables mt, int form, int
   if (i >= n) return;
   const double t = T[i];
   double *o = out + i * NRX;
+  if (!(t > 0.0 && isfinite(t))) {  // ff_log is for positive normal arguments
+    for (int j = 0; j < NRX; ++j) o[j] = CUDART_NAN;
+    return;
+  }
   if (form == 0) {
     GibbsHL g;
     const ff tf = ff_norm(d2ff(t));
