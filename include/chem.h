@@ -320,7 +320,8 @@ typedef struct {
  * NULL).  h_results (nullable, host [max_results]) receives the timed candidates and
  * *n_results their count.
  * cache_path (nullable): a text file of earlier results, one line per key (device name,
- * SM count, variant, max_steps, rtol, atol, floor(log2 ncells), floor(log2 nboxes));
+ * SM count, shape table and mechanism structure, variant, max_steps, rtol, atol,
+ * floor(log2 ncells), floor(log2 nboxes)); lines of another shape table do not match;
  * on a hit *best comes from the file, nothing is launched and *n_results = 0; on a miss
  * the result is appended.  Synchronous; allocates the copies for the duration of the
  * call.  Errors: as chem_integrate_batched; unreadable cache lines are skipped; a cache

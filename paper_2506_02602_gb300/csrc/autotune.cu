@@ -33,8 +33,13 @@ int floor_log2(int64_t v) {
   return l;
 }
 
-// Cache key: device name (spaces as '_'), SM count, variant, max_steps, rtol, atol,
-// floor(log2 ncells), floor(log2 nboxes).
+// The shape table a result's index refers to, raised whenever the entries of kShapeBlock or kShapeMinB
+// (batched.cu) change or their kernels' relative speed does.  Lines of other tables, and those from
+// before there was a mark, do not match.
+constexpr int kShapeTable = 2;
+
+// Cache key: device name (spaces as '_'), SM count, shape table and mechanism structure (species and
+// reactions), variant, max_steps, rtol, atol, floor(log2 ncells), floor(log2 nboxes).
 std::string tune_key(chem_ctx *ctx, double rtol, double atol, int64_t ncells, int64_t nboxes) {
   int dev = 0;
   cudaGetDevice(&dev);
@@ -44,9 +49,9 @@ std::string tune_key(chem_ctx *ctx, double rtol, double atol, int64_t ncells, in
   for (char &c : name)
     if (c == ' ' || c == '\t') c = '_';
   char buf[512];
-  std::snprintf(buf, sizeof buf, "%s %d %d %d %.6e %.6e %d %d", name.c_str(), prop.multiProcessorCount,
-                chem_ctx_variant(ctx), (int)chem_ctx_max_steps(ctx), rtol, atol, floor_log2(ncells),
-                floor_log2(nboxes));
+  std::snprintf(buf, sizeof buf, "%s %d shapes%d/%d/%d %d %d %.6e %.6e %d %d", name.c_str(),
+                prop.multiProcessorCount, kShapeTable, NSP, NRX, chem_ctx_variant(ctx),
+                (int)chem_ctx_max_steps(ctx), rtol, atol, floor_log2(ncells), floor_log2(nboxes));
   return buf;
 }
 
