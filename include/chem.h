@@ -625,7 +625,7 @@ int chem_strang_step(chem_ctx *ctx, const chem_flow1d *flow, int64_t n, double d
 /*
  * Diagnostic: evaluate one of the device math routines the integration kernels use on
  * n fp64 arguments (device pointers d_x -> d_y), so tests can check them against the
- * CUDA library and the IEEE-754 definitions.  op: 0 table-driven exp, 1 table-driven
+ * CUDA library and the IEEE-754 definitions.  op: 0 exp (fixed point for |x| < 700), 1 table-driven
  * log (Tang's methods, used by the kernels), 2 library exp, 3 library log,
  * 4 reciprocal with one Newton-Raphson step, 5 with two, 6 the hardware reciprocal
  * approximation alone, 7 the integer-pipe fp64 -> fp32 rounding (widened back exactly),

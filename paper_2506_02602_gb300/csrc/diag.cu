@@ -17,6 +17,7 @@ namespace chem {
 
 __global__ void k_diag_math(int op, int64_t n, const double *__restrict__ x, double *__restrict__ y) {
   load_math_tables();
+  load_exp2_tables();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double v = x[i];

@@ -40,34 +40,6 @@ __device__ __forceinline__ void load_math_tables() {
   __syncthreads();
 }
 
-// exp(x).  About 1 ulp for x in [-708, 709]: x = (128 m + j) ln2/128 + r, |r| <= ln2/256,
-// e^r - 1 by its degree-5 Taylor polynomial (truncation below 6e-19 relative), and the
-// scale 2^m added to the exponent field of the table entry 2^(j/128) on the integer
-// pipe (10 FP64-pipe operations in all).  Arguments beyond +-710 are first clamped there
-// on the integer pipe, so they still give +inf above and a positive value below 1e-307
-// below, however large; a NaN stays NaN.  Kept out of line, one copy for its many calls.
-static __device__ __noinline__ double exp_t(double x) {
-  const long long kLim = 0x40863000'00000000LL;  // 710.0
-  const long long b = __double_as_longlong(x);
-  const long long ab = b & 0x7fffffffffffffffLL;
-  if (ab > kLim && ab <= 0x7ff0000000000000LL) x = __longlong_as_double((b & (long long)0x8000000000000000ULL) | kLim);
-  const double kShift = 6755399441055744.0;  // 1.5 * 2^52: rounds to an integer in the low bits
-  const double t = fma(x, kInvLn2x128, kShift);
-  const int k = min(max(__double2loint(t), -130816), 130943);  // 2^(k>>7) stays a normal double
-  const double kd = (double)k;
-  double r = fma(-kd, kLn2d128Hi, x);
-  r = fma(-kd, kLn2d128Lo, r);
-  // e^r - 1 = r + r^2/2 + r^3/6 + r^4/24 + r^5/120
-  double p = fma(r, 1.0 / 120.0, 1.0 / 24.0);
-  p = fma(r, p, 1.0 / 6.0);
-  p = fma(r, p, 0.5);
-  p = fma(r, p, 1.0);
-  p = r * p;
-  const double tj = s_exp2_128[k & 127];
-  const double ts = __hiloint2double(__double2hiint(tj) + ((k >> 7) << 20), __double2loint(tj));
-  return fma(ts, p, ts);
-}
-
 // x is a NaN, on the integer pipe
 __device__ __forceinline__ bool is_nan(double x) {
   return (__double_as_longlong(x) & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL;
@@ -121,6 +93,44 @@ __device__ __forceinline__ double exp2_q52_body(long long y) {
 static __device__ __noinline__ double exp2_q52(long long y) { return exp2_q52_body(y); }
 static __device__ __noinline__ double2 exp2_q52(long long y0, long long y1) {
   return make_double2(exp2_q52_body(y0), exp2_q52_body(y1));
+}
+
+// exp(x), about 1 ulp for x in [-708, 709], for the general form of the right-hand side.  |x| < 700:
+// x log2(e) in Q52, rounded (0.6 of its units off), and the exponential above, without FP64
+// instructions.  Beyond, Tang's method: x = (128 m + j) ln2/128 + r, |r| <= ln2/256,
+// e^r - 1 by its degree-5 Taylor polynomial (truncation below 6e-19 relative), and the
+// scale 2^m added to the exponent field of the table entry 2^(j/128) on the integer
+// pipe (10 FP64-pipe operations in all).  Arguments beyond +-710 are first clamped there
+// on the integer pipe, so they still give +inf above and a positive value below 1e-307
+// below, however large; a NaN stays NaN.  Kept out of line, one copy for its many calls.
+static __device__ __noinline__ double exp_t(double x) {
+  const uint32_t ah = (uint32_t)__double2hiint(x) & 0x7fffffffu;
+  if (ah < 0x4085e000u) {  // |x| < 700
+    const unsigned long long m =
+        (((unsigned long long)__double_as_longlong(x) & 0x000fffffffffffffull) | 0x0010000000000000ull) << 11;
+    const unsigned long long q = m >> min(1032 - (int)(ah >> 20), 63);  // |x| in units of 2^-54
+    const long long y = (long long)((__umul64hi(q, kLog2E_q63) + 1) >> 1);
+    return exp2_q52_body(__double2hiint(x) < 0 ? -y : y);
+  }
+  const long long kLim = 0x40863000'00000000LL;  // 710.0
+  const long long b = __double_as_longlong(x);
+  const long long ab = b & 0x7fffffffffffffffLL;
+  if (ab > kLim && ab <= 0x7ff0000000000000LL) x = __longlong_as_double((b & (long long)0x8000000000000000ULL) | kLim);
+  const double kShift = 6755399441055744.0;  // 1.5 * 2^52: rounds to an integer in the low bits
+  const double t = fma(x, kInvLn2x128, kShift);
+  const int k = min(max(__double2loint(t), -130816), 130943);  // 2^(k>>7) stays a normal double
+  const double kd = (double)k;
+  double r = fma(-kd, kLn2d128Hi, x);
+  r = fma(-kd, kLn2d128Lo, r);
+  // e^r - 1 = r + r^2/2 + r^3/6 + r^4/24 + r^5/120
+  double p = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+  p = fma(r, p, 1.0 / 6.0);
+  p = fma(r, p, 0.5);
+  p = fma(r, p, 1.0);
+  p = r * p;
+  const double tj = s_exp2_128[k & 127];
+  const double ts = __hiloint2double(__double2hiint(tj) + ((k >> 7) << 20), __double2loint(tj));
+  return fma(ts, p, ts);
 }
 
 // |x| in units of 2^-Q, truncated, for |x| < 2^(62 - Q + 1).
