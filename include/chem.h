@@ -659,8 +659,8 @@ int chem_diag_fma_peak(int op, int32_t blocks, int32_t threads, int64_t iters, v
  * d_T (device, fp64, kelvin, > 0; values that are not positive and finite give NaN), written to d_out
  * (device, n * n_reactions fp64, row i = temperature i, the fp32 results widened
  * exactly), as the mixed-precision right-hand sides form them: form 0 the mixed
- * variant's (fp64 Gibbs functions summed as fp32 hi/lo pairs), form 1 the all-fp32 one of
- * the surrogate's error test.  The plain fp64 variant forms log2 K_c in fixed point and
+ * variant's (double-float Gibbs functions summed as fp32 hi/lo pairs, before its rounding
+ * test), form 1 the all-fp32 one of the surrogate's error test.  The plain fp64 variant forms log2 K_c in fixed point and
  * has no form here.  Errors: NULL ctx, form not 0 or 1,
  * n outside [0, 2^30] or NULL pointers with n > 0 -> CHEM_ERR_INVALID; a failed launch ->
  * CHEM_ERR_CUDA.  Asynchronous on stream.

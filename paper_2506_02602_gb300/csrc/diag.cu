@@ -15,6 +15,8 @@
 
 namespace chem {
 
+constexpr int kKcBlock = 128;  // threads of k_ln_inv_kc's blocks
+
 __global__ void k_diag_math(int op, int64_t n, const double *__restrict__ x, double *__restrict__ y) {
   load_math_tables();
   load_exp2_tables();
@@ -82,18 +84,28 @@ __global__ void k_fma_coefs(R *ab, R a, R b) {
   ab[1] = b;
 }
 
-template <typename Gibbs, int... J>
-__device__ __forceinline__ void store_ln_inv_kc(const Gibbs &g, double *o, std::integer_sequence<int, J...>) {
+template <int... J>
+__device__ __forceinline__ void store_mixed_exponents(const MixedCols &m, float2 rt, double *o,
+                                                      std::integer_sequence<int, J...>) {
+  auto exponent = [&](int i) {
+    const float2 x = slot_exponent<kKcBlock>(s_rx_row[i], s_rx_k[i].w, rt, m);
+    return (double)fadd(x.x, x.y);
+  };
+  ((o[J] = exponent(rx_slot(J))), ...);
+}
+template <int... J>
+__device__ __forceinline__ void store_f32_exponents(const GibbsF &g, double *o, std::integer_sequence<int, J...>) {
   ((o[J] = (double)ln_inv_kc<J>(g)), ...);
 }
 
-// ln(1 / K_c,j) of every reaction at T[i] into out[i * NRX + j], through the same
-// helpers the right-hand sides call: form 0 the mixed variant's (fp64 Gibbs functions
-// summed as fp32 hi/lo pairs, after the fp64 ln T and 1 / T it takes from the
-// temperature solve), form 1 the error test's all-fp32 one.
-__global__ void k_ln_inv_kc(const __grid_constant__ MechTables mt, int form, int64_t n,
-                            const double *__restrict__ T, double *__restrict__ out) {
-  load_mixed_tables<1>(mt);
+// ln(1 / K_c,j) of every reaction at T[i] into out[i * NRX + j], through the tables, columns and
+// functions of the right-hand sides: form 0 the mixed variant's (double-float ln T and Gibbs
+// functions, summed as fp32 hi/lo pairs, before the rounding test), form 1 the error test's all-fp32
+// one.
+__global__ void __launch_bounds__(kKcBlock)
+    k_ln_inv_kc(const __grid_constant__ MechTables mt, int form, int64_t n, const double *__restrict__ T,
+                double *__restrict__ out) {
+  load_mixed_tables<kKcBlock>(mt);
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double t = T[i];
@@ -102,16 +114,19 @@ __global__ void k_ln_inv_kc(const __grid_constant__ MechTables mt, int form, int
     for (int j = 0; j < NRX; ++j) o[j] = CUDART_NAN;
     return;
   }
+  constexpr auto seq = std::make_integer_sequence<int, NRX>{};
   if (form == 0) {
-    GibbsHL g;
+    const MixedCols m = mixed_cols<kKcBlock>();
+    init_mixed_cols<kKcBlock>(m);
     const ff tf = ff_norm(d2ff(t));
-    gibbs_hl<1>(mt, tf, ff_log(tf), d2ff(rcp1(t)), g.g, g.r);
-    store_ln_inv_kc(g, o, std::make_integer_sequence<int, NRX>{});
+    float2 rt;
+    gibbs_hl<kKcBlock>(mt, tf, ff_log(tf), d2ff(rcp1(t)), m.G, rt);
+    store_mixed_exponents(m, rt, o, seq);
   } else {
     const float tf = (float)t;
     GibbsF g;
     gibbs_f(mt, tf, logf(tf), 1.0f / tf, g);
-    store_ln_inv_kc(g, o, std::make_integer_sequence<int, NRX>{});
+    store_f32_exponents(g, o, seq);
   }
 }
 
@@ -161,10 +176,14 @@ extern "C" int chem_diag_ln_inv_kc(chem_ctx *ctx, int form, int64_t n, const dou
     err = "chem_diag_ln_inv_kc: NULL d_T or d_out";
     return CHEM_ERR_INVALID;
   }
-  const int block = 128;
-  chem::k_ln_inv_kc<<<(unsigned)((n + block - 1) / block), block, 0, (cudaStream_t)stream>>>(
-      chem::chem_ctx_tables(ctx), form, n, d_T, d_out);
-  const cudaError_t e = cudaGetLastError();
+  const int block = chem::kKcBlock;
+  const size_t smem = chem::mixed_cols_bytes(block);
+  cudaError_t e = chem::allow_smem(reinterpret_cast<const void *>(chem::k_ln_inv_kc), smem);
+  if (e == cudaSuccess) {
+    chem::k_ln_inv_kc<<<(unsigned)((n + block - 1) / block), block, smem, (cudaStream_t)stream>>>(
+        chem::chem_ctx_tables(ctx), form, n, d_T, d_out);
+    e = cudaGetLastError();
+  }
   if (e != cudaSuccess) {
     err = std::string("chem_diag_ln_inv_kc: ") + cudaGetErrorString(e);
     return CHEM_ERR_CUDA;

@@ -193,19 +193,15 @@ __device__ __forceinline__ float troe_F_f32(const MechTables &mt, float T, float
 }
 
 // The ingredients of ln(1/K_c,j) = sum_k nu_jk g_k + (sum_k nu_jk) ln(R_u T / p_ref).
-// GibbsHL (mixed variant): g_k / RT and ln(R_u T / p_ref) as fp32 hi/lo pairs; the hi parts
-// sum exactly in fp32 and the lo parts carry the rest, so the fp32 ln(1/K_c) is the sum
-// rounded once (to within ~1e-11); the integrator's loop keeps them in the columns, this
-// struct serves the diagnostics.  GibbsF (the error test's all-fp32 right-hand side): plain fp32.
-struct GibbsHL {
-  float2 g[NGB], r;
-};
+// Mixed variant: g_k / RT (in the columns) and ln(R_u T / p_ref) as fp32 hi/lo pairs; the hi parts
+// sum exactly in fp32 and the lo parts carry the rest (to within ~1e-11).
+// GibbsF (the error test's all-fp32 right-hand side): plain fp32.
 struct GibbsF {
   float g[NSP];
   float r;
 };
 
-// The hi / lo split of a pair for GibbsHL, as split_hilo makes it of an fp64 value: hi = x
+// The hi / lo split of a pair, as split_hilo makes it of an fp64 value: hi = x
 // truncated to a multiple of 2^-12 (for |x| < 2^10, where every g_k above ~70 K lies; a
 // neighbouring multiple beyond), lo the rest.
 __device__ __forceinline__ float2 split_grid(ff x) {
@@ -227,7 +223,7 @@ __device__ __forceinline__ bool ge_mid(const MechTables &mt, ff T) {
 // coefficients pre-combined per range into gc2) of the reactive species and
 // ln(R_u T / p_ref), evaluated in double-float as sums of products with the functions of T
 // (error-free products and two-sums; error ~1e-12 for terms of a few hundred), two species at
-// a time, and split for GibbsHL; species k's parts go to g[k ST].
+// a time, and split; species k's parts go to g[k ST].
 template <int ST>
 __device__ __forceinline__ void gibbs_hl(const MechTables &mt, ff T, ff lnT, ff invT, float2 *g, float2 &r) {
   const int range = ge_mid(mt, T);
@@ -265,18 +261,6 @@ __device__ __forceinline__ void gibbs_f(const MechTables &mt, float T, float lnT
     g.g[k] = fmaf(gc[0], oml, gk);
   }
   g.r = lnT + mt.f.ln_R_over_Pref;
-}
-
-template <int J>
-__device__ __forceinline__ float ln_inv_kc(const GibbsHL &g) {
-  constexpr RxStruct R = kRx[J];
-  constexpr int dnu = n_prod(R) - n_reac(R);
-  float h = g.g[R.p0].x - g.g[R.r0].x, l = g.g[R.p0].y - g.g[R.r0].y;
-  if constexpr (R.p1 >= 0) { h += g.g[R.p1].x; l += g.g[R.p1].y; }
-  if constexpr (R.r1 >= 0) { h -= g.g[R.r1].x; l -= g.g[R.r1].y; }
-  if constexpr (dnu == 1) { h += g.r.x; l += g.r.y; }
-  if constexpr (dnu == -1) { h -= g.r.x; l -= g.r.y; }
-  return h + l;
 }
 
 // Whether x.h + x.l rounds to the same fp32 number anywhere within +-d.
@@ -484,16 +468,23 @@ __device__ __forceinline__ float net_rate(float kf, float lnkf, float t, float2 
   return __fmaf_rn(-fmul(kr, p0), p1, fmul(fmul(kf, r0), r1));
 }
 
-// ln(1 / K_c)'s parts and the net rate of the reaction in slot i (without a third-body
-// factor) into Q, for k_f and its logarithm; returns whether the exponent may round either way.
+// The exponent ln(1 / K_c) of the reaction with rows o and sum nu dn, in two parts.
+template <int ST>
+__device__ __forceinline__ float2 slot_exponent(int4 o, float dn, float2 rt, const MixedCols &m) {
+  const char *g = reinterpret_cast<const char *>(m.G);
+  auto row = [&](int off) { return *reinterpret_cast<const float2 *>(g + off); };
+  return __ffma2_rn(rt, both(dn), sub2(add2(sub2(row(o.z), row(o.x)), row(o.w)), row(o.y)));
+}
+
+// The net rate of the reaction in slot i (without a third-body factor) into Q, for k_f and its
+// logarithm; returns whether the exponent may round either way.
 template <int ST>
 __device__ __forceinline__ bool slot_rate(int i, float kf, float lnkf, float dn, float t, float2 rt, const MixedCols &m) {
-  const char *g = reinterpret_cast<const char *>(m.G);
   constexpr int kC = (NSP + 1) * ST * 8;  // from a row of G to the same row of CU
+  const char *c = reinterpret_cast<const char *>(m.G) + kC;
   const int4 o = s_rx_row[i];
-  auto row = [&](int off) { return *reinterpret_cast<const float2 *>(g + off); };
-  auto conc = [&](int off) { return *reinterpret_cast<const float *>(g + off + kC); };
-  const float2 x = __ffma2_rn(rt, both(dn), sub2(add2(sub2(row(o.z), row(o.x)), row(o.w)), row(o.y)));
+  auto conc = [&](int off) { return *reinterpret_cast<const float *>(c + off); };
+  const float2 x = slot_exponent<ST>(o, dn, rt, m);
   m.Q[i * ST] = net_rate(kf, lnkf, t, x, conc(o.x), conc(o.y), conc(o.z), conc(o.w));
   return !rounds_safely(ff{x.x, x.y}, kLnKcErr);
 }
