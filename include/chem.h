@@ -69,7 +69,7 @@ typedef enum {
                              error (sums of products, exponentials, logarithms; reciprocals
                              by Newton-Raphson refinement of the hardware approximation,
                              within 2 ulp; the temperature solve's steps have an fp32 slope
-                             and end at 4e-9 T, the root exact to ~2e-15) */
+                             and end at 4e-10 T, within 1e-15 of the root) */
   CHEM_VARIANT_MIXED = 1  /* rates and RK stage derivatives in fp32; solution and error
                              registers and step control in fp64; temperature solve and Gibbs
                              functions in double-float, redone in fp64 where the fp32 rounding

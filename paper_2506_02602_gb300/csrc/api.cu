@@ -3,6 +3,7 @@
 // launches on the caller's stream, the host-buffer convenience path, error strings.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -213,7 +214,8 @@ int build_tables(const chem_mechanism *m, MechTables *t) {
     t->eff_mask[j] = mask;
   }
   // fixed-point forms: every sum of products below stays inside 64 bits for T in (128, 8192) K,
-  // |Y| < 1.25 and rho in (2^-64, 2^64) when the magnitudes here are below their bounds
+  // |Y| < 1.25, sum |Y| <= 1.5, |e/R| < 2^26 and rho in (2^-64, 2^64) when the magnitudes here are
+  // below their bounds
   const double log2e = 1.4426950408889634;
   t->fixed_ok = Tmid > 128.0 && Tmid < 8192.0;
   auto qcoef = [](double v, int q, int drop) {
@@ -242,16 +244,36 @@ int build_tables(const chem_mechanism *m, MechTables *t) {
   }
   for (int r = 0; r < 2 && t->fixed_ok; ++r) {
     int S = 13;
-    if (r == 0) while (std::ldexp(1.0, S - 1) >= Tmid) --S;
+    if (r == 0) while (std::ldexp(1.0, S - 1) > 1.000001 * Tmid) --S;  // t < 1 - 2^-20
     t->q_log2[r] = S;
-    double esum = 0.0, ei[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    // the energies: the finest unit 2^-Q that holds the coefficients (Q + 2), the cross sums
+    // (sum_k |v_ki| 2^Q + 2^61) and Horner's sums with e/R
+    double emax = 0.0, erow = 0.0, ei[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    auto evalue = [&](int k, int i) { return i < 5 ? std::ldexp(t->ecw[r][k][i], S * (i + 1)) : t->ecw[r][k][5]; };
+    for (int k = 0; k < NSP; ++k) {
+      double row = 0.0;
+      for (int i = 0; i < 6; ++i) {
+        const double v = std::fabs(evalue(k, i));
+        ei[i] += v;
+        row += v;
+        emax = std::fmax(emax, v);
+      }
+      erow = std::fmax(erow, row);
+    }
+    const double ecol = *std::max_element(ei, ei + 6);
+    int Q = 37;
+    while (Q >= 33 && !(std::ldexp(emax, Q + 2) < 0x1.fp62 && std::ldexp(ecol, Q) < 0x1.8p62 &&
+                        std::ldexp(1.5 * erow + 0x1p26, Q) < 0x1.fp62))
+      --Q;
+    if (Q < 33) {
+      t->fixed_ok = 0;
+      break;
+    }
+    t->q_res[r] = Q;
     for (int k = 0; k < NSP; ++k) {
       for (int i = 0; i < 6; ++i) {
-        const double v = i < 5 ? std::ldexp(t->ecw[r][k][i], S * (i + 1)) : t->ecw[r][k][5];
-        ei[i] += std::fabs(v);
-        esum += std::fabs(v);
-        if (std::fabs(v) < 0x1p26) t->qe[r][k][i] = qcoef(v, 37, 2);
-        else t->fixed_ok = 0;
+        const int64_t x = (int64_t)std::llrint(std::ldexp(evalue(k, i), Q + 2));
+        t->qe[r][k][i] = {(int32_t)((x + 0x80000000ll) >> 32), (int32_t)(uint32_t)x >> 1};
       }
       const double *g = t->gc[r][k];
       double gsum = 13.0 * std::fabs(g[0]) + std::fabs(g[5]) * log2e / 128.0 + std::fabs(g[0] + g[6]) * log2e;
@@ -271,9 +293,6 @@ int build_tables(const chem_mechanism *m, MechTables *t) {
       for (int i = 0; i < 4; ++i) t->qgt[r][k][i] = qcoef(gt[i], 57, 4);
       t->qg1[r][k] = (int64_t)std::ldexp(-log2e * (g[0] + g[6]), 50);
     }
-    for (int i = 0; i < 6; ++i)
-      if (!(ei[i] < 0x1p26 * 1.4)) t->fixed_ok = 0;
-    if (!(esum < 0x1.4p28 * 1.1)) t->fixed_ok = 0;
   }
   if (t->fixed_ok) t->qT_mid = (int64_t)std::ldexp(Tmid, 50);
   t->qRP = (int64_t)std::ldexp(std::log2(R_U / P_REF), 50);

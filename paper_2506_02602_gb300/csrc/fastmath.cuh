@@ -167,6 +167,13 @@ struct Limbs { int h, l; };
 template <int D>
 __device__ __forceinline__ Limbs<D> limbs(long long v) { return {(int)(v >> 32), (int)((uint32_t)v >> D)}; }
 
+// The same with the lower half in [-2^31, 2^31) and its limb signed, so that what is dropped has no
+// bias.  v + 2^31 must not overflow.
+template <int D>
+__device__ __forceinline__ Limbs<D> limbs_centred(long long v) {
+  return {(int)((unsigned long long)v >> 32) + (int)((uint32_t)v >> 31), (int)(uint32_t)v >> D};
+}
+
 template <int D>
 struct DotQ {
   long long h, x;
@@ -176,6 +183,11 @@ struct DotQ {
     x += (long long)cl * p.h;
   }
   __device__ __forceinline__ long long value() const { return h + (x >> (32 - D)); }  // sum / 2^64
+  // the same modulo 2^64 with F more bits
+  template <int F>
+  __device__ __forceinline__ unsigned long long fine() const {
+    return ((unsigned long long)h << F) + (unsigned long long)(x >> (32 - D - F));
+  }
 };
 
 // m t 2^-63 for 0 <= t < 2^63
@@ -183,6 +195,22 @@ __device__ __forceinline__ long long mul_q63(long long m, long long t) {
   const int mh = (int)(m >> 32), ml = (int)((uint32_t)m >> 1), th = (int)(t >> 32), tl = (int)((uint32_t)t >> 1);
   return (((long long)mh * th) << 1) + (((long long)mh * tl + (long long)ml * th) >> 30);
 }
+
+// The same from centred limbs, rounded; fine() is modulo 2^64, with F more bits.
+struct MulQ {
+  long long h, x;
+  __device__ __forceinline__ MulQ(long long m, const Limbs<1> &t) {
+    const Limbs<1> a = limbs_centred<1>(m);
+    h = (long long)a.h * t.h;
+    x = (long long)a.h * t.l + (1ll << 29);
+    x += (long long)a.l * t.h;
+  }
+  __device__ __forceinline__ long long value() const { return (h << 1) + (x >> 30); }
+  template <int F>
+  __device__ __forceinline__ unsigned long long fine() const {
+    return ((unsigned long long)h << (1 + F)) + (unsigned long long)((x - (1ll << 29)) >> (30 - F));
+  }
+};
 
 // Per-block copies of k_log2_c and k_log2_q58, filled by load_log2_table().
 __shared__ unsigned short s_log2_c[256];

@@ -66,7 +66,8 @@ struct MechTablesF32 {
   float T_mid2[2], ln_R_over_Pref2[2];
 };
 
-// A coefficient in fixed point: h 2^32 plus the top bits l of the lower half (2^2 l, or 2^4 l in qgt)
+// A coefficient in fixed point: h 2^32 plus the top bits l of the lower half (2^2 l, or 2^4 l in qgt;
+// in qe the lower half is signed and its limb 2 l)
 struct QCoef { int32_t h, l; };
 
 // Per-context tables (host-built from chem_mechanism by build_tables()).
@@ -96,13 +97,13 @@ struct MechTables {
   int64_t qA[NRX], qA0[NRX];
   QCoef qB[NRX], qH[NRX], qB0[NRX], qH0[NRX];
   double troe_q3[NRX], troe_q1[NRX], troe_q2[NRX];
-  // t = T 2^-S per range, S = q_log2[range]: ecw (Q37) times 2^(S (i+1)), the Gibbs functions
+  // t = T 2^-S per range, S = q_log2[range]: ecw (Q q_res + 2) times 2^(S (i+1)), the Gibbs functions
   // times -log2(e) by log2 T (Q56), 1/T (Q44), t .. t^4 (Q57) and 1 (Q50)
   QCoef qe[2][NSP][6];
   QCoef qg[2][NSP][2], qgt[2][NSP][4];
   int64_t qg1[2][NSP];
   int64_t qT_mid, qRP;  // T_mid (Q50), log2(R_u / p_ref) (Q50)
-  int32_t q_log2[2];
+  int32_t q_log2[2], q_res[2];
   int32_t fixed_ok;
   // third-body efficiencies minus one: [M] = sum_k c_k + sum_k effm1 c_k
   double effm1[NRX][NSP];

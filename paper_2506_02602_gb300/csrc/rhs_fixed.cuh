@@ -7,8 +7,8 @@
 // logarithms are sums of products in 64-bit fixed point (DotQ: 15 cycles a term), which keep more
 // digits than fp64 where terms cancel (Gibbs functions of a few hundred have an fp64 rounding
 // error of 2^-46, here 2^-50), and the exponentials follow in exp2_q52.
-//   - Newton on e(T) evaluates the residual in units of 2^-33 of e / R_u (fp64 rounds the sums of
-//     magnitude 1e6 it has there to 2^-33) and divides it by an fp32 c_v: the step is then off by
+//   - Newton on e(T) evaluates the residual in units down to 2^-40 of e / R_u (fp64 rounds the sums
+//     of magnitude 1e6 it has there to 2^-33) and divides it by an fp32 c_v: the step is then off by
 //     ~2^-21 of itself, and the iteration goes on until that no longer counts.
 //   - Concentrations are per mass (y_k = Y_k / W_k); the powers of rho that belong to the rates
 //     enter as log2(rho) in their exponents.
@@ -17,11 +17,12 @@
 //     of one stoichiometry (duplicates, colliders) share it with their k_f summed.
 // A warp's evaluation issued 1040 FP64 instructions in the general form, 637 with only its
 // exponentials in fixed point and 300 here; the 1M-cell detonation slice takes 83.2, 49.2 and
-// 26.1 ms, a 256-cell batch of 15 steps 3.0, 2.1 and 1.5 ms (one warp's chain of dependent
+// 24.9 ms, a 256-cell batch of 15 steps 3.0, 2.1 and 1.3 ms (one warp's chain of dependent
 // instructions).  Integer work now fills the issue slots the FP64 pipe (70 % busy) leaves.
 //
-// For T in (128, 8192) K, |Y_k| < 1.25, rho in (2^-64, 2^64) and coefficients within the
-// tables' ranges (MechTables::fixed_ok); anything else takes the general form (rhs.cuh).
+// For T in (128, 8192) K, |Y_k| < 1.25, sum |Y_k| <= 1.5, |e| / R_u < 2^26 K mol/kg, rho in
+// (2^-64, 2^64) and coefficients within the tables' ranges (MechTables::fixed_ok); anything else takes
+// the general form (rhs.cuh).
 #pragma once
 
 #include <utility>
@@ -83,9 +84,9 @@ __device__ __forceinline__ void load_fixed_tables(const MechTables &mt) {
 
 constexpr int kRoll = 3;  // species of a rolled loop's step
 
-// 128 < T < 8192 and 2^-64 < rho < 2^64, on the high words
+// 128 < T < 8191.996 and 2^-64 < rho < 2^64, on the high words
 __device__ __forceinline__ bool fixed_T(double T) {
-  return (uint32_t)__double2hiint(T) - 0x40600001u < 0x40c00000u - 0x40600001u;
+  return (uint32_t)__double2hiint(T) - 0x40600001u < 0x40bfffffu - 0x40600001u;
 }
 __device__ __forceinline__ bool fixed_rho(double rho) {
   return (uint32_t)__double2hiint(rho) - 0x3bf00000u < 0x43f00000u - 0x3bf00000u;
@@ -93,34 +94,43 @@ __device__ __forceinline__ bool fixed_rho(double rho) {
 
 // Temperature from (e, Y) as solve_T: the same iteration from the same guess.  False when an
 // argument is out of range or an iterate leaves it, or without convergence; T is then unchanged.
-// The step's fp32 slope leaves 2^-21 of it, so the iteration stops at dT <= 4e-9 T with T exact
-// to 2e-15: one iteration more than solve_T, but of 300 cycles where solve_T's take 850.
+//
+// The residual is in units of 2^-q_res of e/R_u (2^-36 below T_mid and 2^-35 above for the mechanisms
+// here).  Sums are rounded and the limbs centred, so that what is dropped does not add up, and where
+// the residual is small (2^9 at most) its last multiplication and its constant term keep 4 more bits,
+// modulo 2^64.  So T is within 7e-16 of the root (rms 1e-16 to 1.6e-16), as in
+// fp64; with units of 2^-33 and everything truncated it was off by up to 4e-14 (rms 1e-15 to 1e-14).
+// The step's fp32 slope leaves 2^-21 of it; a step of 4e-10 T ends the iteration.
 template <int ST>
 __device__ __forceinline__ bool solve_T_fixed(const MechTables &mt, const double *U, double eR, double &T) {
-  if (!fixed_T(T) || ((uint32_t)__double2hiint(eR) & 0x7fffffffu) >= 0x41b00000u) return false;  // |eR| < 2^28
-  const long long sg = (long long)__double2hiint(eR) >> 31;
-  const long long eq = ((long long)abs_q<33>(eR) ^ sg) - sg;
+  constexpr int kFine = 4;
+  const uint32_t eh = (uint32_t)__double2hiint(eR) & 0x7fffffffu;
+  if (!fixed_T(T) || eh >= 0x41900000u) return false;  // |eR| < 2^26
   long long Tq = (long long)abs_q<50>(T);
   long long m[6];
+  unsigned long long m5f = 0;
   float d[5];
   int range = -1, shift = 0;
   float unit = 0.0f;
+  bool done = false;
   for (int it = 0; it < 30; ++it) {
     const int r = Tq >= mt.qT_mid;
     if (r != range) {  // mixture coefficients
       range = r;
       shift = 13 - mt.q_log2[r];
       unit = __int_as_float((127 + 13 - shift) << 23);
-      DotQ<2> s[6];
+      DotQ<1> s[6];
 #pragma unroll
-      for (int i = 0; i < 6; ++i) s[i] = {0, 0};
-      uint32_t big = 0;
+      for (int i = 0; i < 6; ++i) s[i] = {0, i < 5 ? 1ll << 30 : 0};  // halves: the values are rounded
+      uint32_t big = 0, sum = 0;
 #pragma unroll kRoll
       for (int k = 0; k < NSP; ++k) {
         const double yk = U[k * ST];
         big = max(big, (uint32_t)__double2hiint(yk) & 0x7fffffffu);
         const long long sy = (long long)__double2hiint(yk) >> 31;
-        const Limbs<2> y = limbs<2>(((long long)abs_q<60>(yk) ^ sy) - sy);
+        const long long ay = (long long)abs_q<62>(yk);
+        sum += (uint32_t)(ay >> 36);
+        const Limbs<1> y = limbs_centred<1>((ay ^ sy) - sy);
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
           const int4 q = s_qe[r][k][i];
@@ -128,31 +138,44 @@ __device__ __forceinline__ bool solve_T_fixed(const MechTables &mt, const double
           s[2 * i + 1].add(q.z, q.w, y);
         }
       }
-      if (big >= 0x3ff40000u) return false;  // |Y| < 1.25
+      if (big >= 0x3ff40000u || sum > 0x06000000u - NSP) break;  // |Y| < 1.25, sum |Y| <= 1.5
 #pragma unroll
       for (int i = 0; i < 6; ++i) m[i] = s[i].value();
-      m[5] -= eq;
+      m5f = s[5].template fine<kFine>();
+      {  // e/R_u, truncated
+        const int n = (int)(eh >> 20) - 1075 + mt.q_res[r];
+        const unsigned long long a =
+            ((unsigned long long)__double_as_longlong(eR) & 0x000fffffffffffffull) | 0x0010000000000000ull;
+        const unsigned long long c = n >= 0 ? a << n : a >> min(-n, 63);
+        const unsigned long long f = n + kFine >= 0 ? a << (n + kFine) : a >> min(-n - kFine, 63);
+        const bool neg = __double2hiint(eR) < 0;
+        m[5] -= neg ? -(long long)c : (long long)c;
+        m5f -= neg ? 0ull - f : f;
+      }
 #pragma unroll
       for (int i = 0; i < 5; ++i) d[i] = (float)(i + 1) * __ll2float_rn(m[i]);
     }
     const long long t = Tq << shift;
+    const Limbs<1> tl = limbs_centred<1>(t);
     long long e = m[4];
 #pragma unroll
-    for (int i = 3; i >= 0; --i) e = mul_q63(e, t) + m[i];
-    e = mul_q63(e, t) + m[5];
+    for (int i = 3; i >= 0; --i) e = MulQ(e, tl).value() + m[i];
+    const MulQ p(e, tl);
+    e = p.value() + m[5];
+    const bool fine = (uint32_t)(int)(e >> 32) + 0x1000u < 0x2000u;  // |e| < 2^44: a few K at most
+    if (fine) e = (long long)(p.template fine<kFine>() + m5f);
     const float tf = __ll2float_rn(t) * 0x1p-63f;
     const float cv = fmaf(tf, fmaf(tf, fmaf(tf, fmaf(tf, d[4], d[3]), d[2]), d[1]), d[0]);
-    const float dT = __fdividef(__ll2float_rn(e), cv) * unit;
-    if (!(fabsf(dT) < 4096.0f)) return false;
+    const float dT = __fdividef(__ll2float_rn(e), cv) * (fine ? unit * (1.0f / (1 << kFine)) : unit);
+    if (!(fabsf(dT) < 4096.0f)) break;
     Tq -= __float2ll_rn(dT * 0x1p50f);
-    if ((uint32_t)(Tq >> 32) - 0x02000001u >= 0x80000000u - 0x02000001u) return false;
+    if ((uint32_t)(Tq >> 32) - 0x02000001u >= 0x7fffffffu - 0x02000001u) break;
     const float Tf = (float)(int)(Tq >> 32) * 0x1p-18f;
-    if (fabsf(dT) <= 4e-9f * Tf) {
-      T = q50_to_double(Tq);
-      return true;
-    }
+    done = fine && fabsf(dT) <= 4e-10f * Tf;
+    if (done) break;
   }
-  return false;
+  if (done) T = q50_to_double(Tq);
+  return done;
 }
 
 struct RateInputsQ {
