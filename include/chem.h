@@ -638,6 +638,14 @@ int chem_strang_step(chem_ctx *ctx, const chem_flow1d *flow, int64_t n, double d
 int chem_diag_math(int op, int64_t n, const double *d_x, double *d_y, void *stream);
 
 /*
+ * Diagnostic: the same for the fixed-point routines of the fp64 kernel.  op: 0 2^x (|x| < 1021, x
+ * first rounded to a multiple of 2^-52), 1 / 2 log2 x as a 64-bit integer in d_y's bits, in units of
+ * 2^-58 (x in (2^-31, 2^31)) and of 2^-52 (x positive and normal), 3 the reciprocal by one third-order
+ * step.  Errors and stream as chem_diag_math.
+ */
+int chem_diag_fixed_math(int op, int64_t n, const double *d_x, double *d_y, void *stream);
+
+/*
  * Diagnostic: a throughput probe of the FMA pipe the integration kernels are bound by
  * (the denominator of their compute roofline; the paper has no counterpart).  op 0:
  * fp64, 1: fp32.  Launches blocks x threads threads; each runs iters rounds of 32 FMAs

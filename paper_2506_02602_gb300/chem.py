@@ -144,6 +144,7 @@ def load(n_species: int = 9) -> C.CDLL:
         "chem_integrate": (C.c_int, [vp, C.POINTER(State), i64, dbl, dbl, dbl, vp, vp]),
         "chem_integrate_host": (C.c_int, [vp, i64, vp, vp, vp, i64, vp, vp, vp, vp, dbl, dbl, dbl, vp]),
         "chem_diag_math": (C.c_int, [C.c_int, i64, vp, vp, vp]),
+        "chem_diag_fixed_math": (C.c_int, [C.c_int, i64, vp, vp, vp]),
         "chem_diag_fma_peak": (C.c_int, [C.c_int, C.c_int32, C.c_int32, i64, vp, vp]),
         "chem_diag_ln_inv_kc": (C.c_int, [vp, C.c_int, i64, vp, vp, vp]),
         "chem_integrate_batched": (C.c_int, [vp, C.POINTER(State), i64, C.POINTER(Batch), dbl, dbl,
@@ -190,6 +191,18 @@ def diag_math(op: int, x, stream=None):
     rc = load().chem_diag_math(op, x.numel(), _ptr(x), _ptr(y), _stream(stream))
     if rc != OK:
         raise ChemError(rc, "chem_diag_math failed")
+    return y
+
+
+def diag_fixed_math(op: int, x, stream=None):
+    """chem_diag_fixed_math on a float64 CUDA tensor; returns a new tensor.  op: 0 fixed-point 2^x,
+    1 / 2 log2 as int64 bits in units of 2^-58 / 2^-52, 3 third-order reciprocal."""
+    import torch
+    _check_f64_cuda("x", x)
+    y = torch.empty_like(x)
+    rc = load().chem_diag_fixed_math(op, x.numel(), _ptr(x), _ptr(y), _stream(stream))
+    if rc != OK:
+        raise ChemError(rc, "chem_diag_fixed_math failed")
     return y
 
 

@@ -1,5 +1,6 @@
-// diag.cu -- diagnostics: chem_diag_math (the kernels' device math routines on caller
-// arrays, for accuracy tests against the CUDA library and the IEEE-754 definitions),
+// diag.cu -- diagnostics: chem_diag_math and chem_diag_fixed_math (the kernels' device math
+// routines on caller arrays, for accuracy tests against the CUDA library, extended precision and the
+// IEEE-754 definitions),
 // chem_diag_fma_peak (an FMA-throughput probe of the fp64 and fp32 pipes, the
 // denominators of the integrators' compute roofline) and chem_diag_ln_inv_kc (the
 // equilibrium exponents as the mixed-precision right-hand sides form them).
@@ -51,6 +52,19 @@ __global__ void k_diag_math(int op, int64_t n, const double *__restrict__ x, dou
     }
   }
   y[i] = r;
+}
+
+// The fixed-point routines of the fp64 kernel.
+__global__ void k_diag_fixed_math(int op, int64_t n, const double *__restrict__ x, double *__restrict__ y) {
+  load_exp2_tables();
+  load_log2_table();
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double v = x[i];
+  if (op == 0) y[i] = exp2_q52(__double2ll_rn(v * 0x1p52));
+  else if (op == 1) y[i] = __longlong_as_double(log2_q58(v));
+  else if (op == 2) y[i] = __longlong_as_double(log2_q52(v));
+  else y[i] = rcp3(v);
 }
 
 // FMA-pipe throughput probe: 8 independent dependent chains per thread, x <- x a + b,
@@ -159,6 +173,15 @@ extern "C" int chem_diag_math(int op, int64_t n, const double *d_x, double *d_y,
   if (!d_x || !d_y) return CHEM_ERR_INVALID;
   const int block = 256;
   chem::k_diag_math<<<(unsigned)((n + block - 1) / block), block, 0, (cudaStream_t)stream>>>(op, n, d_x, d_y);
+  return cudaGetLastError() == cudaSuccess ? CHEM_OK : CHEM_ERR_CUDA;
+}
+
+extern "C" int chem_diag_fixed_math(int op, int64_t n, const double *d_x, double *d_y, void *stream) {
+  if (op < 0 || op > 3 || n < 0) return CHEM_ERR_INVALID;
+  if (n == 0) return CHEM_OK;
+  if (!d_x || !d_y) return CHEM_ERR_INVALID;
+  const int block = 256;
+  chem::k_diag_fixed_math<<<(unsigned)((n + block - 1) / block), block, 0, (cudaStream_t)stream>>>(op, n, d_x, d_y);
   return cudaGetLastError() == cudaSuccess ? CHEM_OK : CHEM_ERR_CUDA;
 }
 

@@ -73,17 +73,21 @@ __device__ __forceinline__ void load_exp2_tables() {
 
 __device__ __forceinline__ unsigned long long mul_wide(uint32_t a, uint32_t b) { return (unsigned long long)a * b; }
 
-// 2^(y 2^-52) for |y| < 1021 2^52
-__device__ __forceinline__ double exp2_q52_body(long long y) {
+// 2^(y 2^-52 + yx 2^-84) for |y| < 1021 2^52; yx = 0 unless kLong
+template <bool kLong = false>
+__device__ __forceinline__ double exp2_q52_body(long long y, uint32_t yx = 0) {
   const uint32_t yl = (uint32_t)y, yh = (uint32_t)(y >> 32);
   const unsigned long long t = s_exp2_hi[(yh >> 10) & 1023], s0 = s_exp2_lo[yh & 1023];
-  const unsigned long long v = mul_wide(yl, kLn2Q64Hi) + __umulhi(yl, kLn2Q64Lo);  // units of 2^-84
+  unsigned long long v = mul_wide(yl, kLn2Q64Hi) + __umulhi(yl, kLn2Q64Lo);  // units of 2^-84
+  if constexpr (kLong) v += __umulhi(yx, kLn2Q64Hi);
   const uint32_t vh = (uint32_t)(v >> 32);
   const unsigned long long w = v + mul_wide(__umulhi(vh, vh), 2048u);  // + v^2/2
   // (1 + s0) (1 + w) - 1 in units of 2^-64
   const unsigned long long s = s0 + (w >> 20) + mul_wide(__umulhi((uint32_t)(s0 >> 22), (uint32_t)(w >> 32)), 4u);
   const uint32_t th = (uint32_t)(t >> 32), tl = (uint32_t)t, sh = (uint32_t)(s >> 32), sl = (uint32_t)s;
-  const unsigned long long p = (t + mul_wide(th, sh) + __umulhi(th, sl) + __umulhi(tl, sh)) >> 11;  // 53 bits, rounded
+  const unsigned long long u = t + mul_wide(th, sh) + __umulhi(th, sl) + __umulhi(tl, sh);
+  unsigned long long p = u >> 11;  // 53 bits, rounded
+  if constexpr (kLong) p |= (unsigned long long)(u < t) << 53;  // less than half an ulp below the next power of 2
   // the leading bit, or a carry, adds to the exponent
   return __hiloint2double((int)((uint32_t)(p >> 32) + (yh & 0xfff00000u) + (1022u << 20)), (int)(uint32_t)p);
 }
@@ -95,9 +99,9 @@ static __device__ __noinline__ double2 exp2_q52(long long y0, long long y1) {
   return make_double2(exp2_q52_body(y0), exp2_q52_body(y1));
 }
 
-// exp(x), about 1 ulp for x in [-708, 709], for the general form of the right-hand side.  |x| < 700:
-// x log2(e) in Q52, rounded (0.6 of its units off), and the exponential above, without FP64
-// instructions.  Beyond, Tang's method: x = (128 m + j) ln2/128 + r, |r| <= ln2/256,
+// exp(x) for the general form of the right-hand side.  |x| < 700: x log2(e) in units of 2^-84 from a
+// 128-bit product and the exponential above, 0.51 ulp, without FP64 instructions.  Beyond, Tang's
+// method, about 1 ulp: x = (128 m + j) ln2/128 + r, |r| <= ln2/256,
 // e^r - 1 by its degree-5 Taylor polynomial (truncation below 6e-19 relative), and the
 // scale 2^m added to the exponent field of the table entry 2^(j/128) on the integer
 // pipe (10 FP64-pipe operations in all).  Arguments beyond +-710 are first clamped there
@@ -108,9 +112,16 @@ static __device__ __noinline__ double exp_t(double x) {
   if (ah < 0x4085e000u) {  // |x| < 700
     const unsigned long long m =
         (((unsigned long long)__double_as_longlong(x) & 0x000fffffffffffffull) | 0x0010000000000000ull) << 11;
-    const unsigned long long q = m >> min(1032 - (int)(ah >> 20), 63);  // |x| in units of 2^-54
-    const long long y = (long long)((__umul64hi(q, kLog2E_q63) + 1) >> 1);
-    return exp2_q52_body(__double2hiint(x) < 0 ? -y : y);
+    const int n = 1033 - (int)(ah >> 20);  // m = |x| 2^(53 + n), n >= 1
+    const unsigned long long p = m * kLog2E_q127Hi, lo = p + __umul64hi(m, kLog2E_q127Lo);
+    const unsigned long long hi = __umul64hi(m, kLog2E_q127Hi) + (lo < p);
+    long long y = n < 64 ? (long long)(hi >> n) : 0;
+    uint32_t yx = n < 64 ? (uint32_t)(((hi << (64 - n)) | (lo >> n)) >> 32) : (uint32_t)(hi >> min(n - 32, 63));
+    if (__double2hiint(x) < 0) {
+      y = -y - (yx != 0u);
+      yx = 0u - yx;
+    }
+    return exp2_q52_body<true>(y, yx);
   }
   const long long kLim = 0x40863000'00000000LL;  // 710.0
   const long long b = __double_as_longlong(x);

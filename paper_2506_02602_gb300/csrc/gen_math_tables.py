@@ -110,7 +110,8 @@ def main():
         f"constexpr double kLog2E = {hexd(1 / LN2)}, kLog2_10 = {hexd(Decimal(10).ln() / LN2)};",
         f"constexpr unsigned kLn2Q64Hi = {int(LN2 * 2**64) >> 32:#x}u, kLn2Q64Lo = {int(LN2 * 2**64) & 0xffffffff:#x}u;",
         f"constexpr long long kLog2E_q62 = {int((1 / LN2 * 2**62).to_integral_value()):#x}ll;",
-        f"constexpr unsigned long long kLog2E_q63 = {int((1 / LN2 * 2**63).to_integral_value()):#x}ull;",
+        f"constexpr unsigned long long kLog2E_q127Hi = {int(1 / LN2 * 2**127) >> 64:#x}ull, "
+        f"kLog2E_q127Lo = {int(1 / LN2 * 2**127) & (2**64 - 1):#x}ull;",
         f"constexpr long long kLog2EThird_q64 = {int((1 / LN2 / 3 * 2**64).to_integral_value()):#x}ll;",
         f"constexpr float kLn2A = {ln2a.hex()}f, kLn2B = {ln2b.hex()}f, kLn2C = {ln2c.hex()}f;",
         f"constexpr double kLn10 = {hexd(Decimal(10).ln())};",
