@@ -638,10 +638,11 @@ int chem_strang_step(chem_ctx *ctx, const chem_flow1d *flow, int64_t n, double d
 int chem_diag_math(int op, int64_t n, const double *d_x, double *d_y, void *stream);
 
 /*
- * Diagnostic: the same for the fixed-point routines of the fp64 kernel.  op: 0 2^x (|x| < 1021, x
- * first rounded to a multiple of 2^-52), 1 / 2 log2 x as a 64-bit integer in d_y's bits, in units of
- * 2^-58 (x in (2^-31, 2^31)) and of 2^-52 (x positive and normal), 3 the reciprocal by one third-order
- * step.  Errors and stream as chem_diag_math.
+ * Diagnostic: the same for the fixed-point routines of the fp64 kernel and the double-float
+ * logarithm of the mixed one.  op: 0 2^x (|x| < 1021, x first rounded to a multiple of 2^-52),
+ * 1 / 2 log2 x as a 64-bit integer in d_y's bits, in units of 2^-58 (x in (2^-31, 2^31)) and of
+ * 2^-52 (x positive and normal), 3 the reciprocal by one third-order step, 4 the double-float ln x
+ * (x in fp32's normal range, first rounded to a pair).  Errors and stream as chem_diag_math.
  */
 int chem_diag_fixed_math(int op, int64_t n, const double *d_x, double *d_y, void *stream);
 

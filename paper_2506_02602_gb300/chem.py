@@ -196,7 +196,7 @@ def diag_math(op: int, x, stream=None):
 
 def diag_fixed_math(op: int, x, stream=None):
     """chem_diag_fixed_math on a float64 CUDA tensor; returns a new tensor.  op: 0 fixed-point 2^x,
-    1 / 2 log2 as int64 bits in units of 2^-58 / 2^-52, 3 third-order reciprocal."""
+    1 / 2 log2 as int64 bits in units of 2^-58 / 2^-52, 3 third-order reciprocal, 4 double-float ln."""
     import torch
     _check_f64_cuda("x", x)
     y = torch.empty_like(x)

@@ -54,17 +54,23 @@ __global__ void k_diag_math(int op, int64_t n, const double *__restrict__ x, dou
   y[i] = r;
 }
 
-// The fixed-point routines of the fp64 kernel.
+// The fixed-point routines of the fp64 kernel, and the mixed kernel's double-float logarithm.
 __global__ void k_diag_fixed_math(int op, int64_t n, const double *__restrict__ x, double *__restrict__ y) {
   load_exp2_tables();
   load_log2_table();
+  load_ln_ff();
+  __syncthreads();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double v = x[i];
   if (op == 0) y[i] = exp2_q52(__double2ll_rn(v * 0x1p52));
   else if (op == 1) y[i] = __longlong_as_double(log2_q58(v));
   else if (op == 2) y[i] = __longlong_as_double(log2_q52(v));
-  else y[i] = rcp3(v);
+  else if (op == 3) y[i] = rcp3(v);
+  else {
+    const ff t = ff_log(ff_norm(d2ff(v)));
+    y[i] = (double)t.h + (double)t.l;
+  }
 }
 
 // FMA-pipe throughput probe: 8 independent dependent chains per thread, x <- x a + b,
@@ -177,7 +183,7 @@ extern "C" int chem_diag_math(int op, int64_t n, const double *d_x, double *d_y,
 }
 
 extern "C" int chem_diag_fixed_math(int op, int64_t n, const double *d_x, double *d_y, void *stream) {
-  if (op < 0 || op > 3 || n < 0) return CHEM_ERR_INVALID;
+  if (op < 0 || op > 4 || n < 0) return CHEM_ERR_INVALID;
   if (n == 0) return CHEM_OK;
   if (!d_x || !d_y) return CHEM_ERR_INVALID;
   const int block = 256;

@@ -154,8 +154,8 @@ __device__ __forceinline__ void load_mixed_tables(const MechTables &mt) {
       for (int q = 0; q < 7; ++q) s_gc[r][k / 2][q] = make_float4(g[q][0], g1[q][0], g[q][1], g1[q][1]);
     }
   }
+  load_ln_ff();
   for (int i = threadIdx.x; i < 65; i += blockDim.x) {
-    s_ln_ff[i] = make_float4(k_ln_ff[i][0], k_ln_ff[i][1], k_ln_ff[i][2], 0.0f);
     s_log_inv[i] = k_log_inv[i];
     s_log_tab[i] = k_log_tab[i];
     s_log_tab_m1[i] = k_log_tab_m1[i];

@@ -7,6 +7,9 @@
 * log2 in units of 2^-58: 6 units, at the edges of its 256 intervals; in units of 2^-52 over the whole
   range of fp64, one unit (truncation) more;
 * reciprocal: 2 ulp.
+
+And the mixed kernel's double-float ln for |ln x| < 16: the roundings of low parts of at most 2^-21, six
+of them, 6 x 2^-46.
 """
 import numpy as np
 import pytest
@@ -82,3 +85,17 @@ def test_reciprocal():
     err = _ulps(_math(3, x), 1 / x.astype(L))
     print(f"\nreciprocal: {float(err.max()):.3f} ulp")
     assert err.max() <= 2.0
+
+
+def test_double_float_log():
+    rng = np.random.default_rng(25)
+    j = 1.0 + (np.arange(65) - 0.5) / 64.0  # the table's interval edges
+    f = np.concatenate([j[1:], np.nextafter(j[1:].astype(np.float32), np.float32(0)).astype(np.float64),
+                        1.0 + np.arange(64) / 64.0])
+    x = np.concatenate([rng.uniform(100.0, 9000.0, 200000), np.exp(rng.uniform(-15.9, 15.9, 100000)),
+                        *(f * 2.0**e for e in (-20, -1, 0, 8, 12)), 1.0 + np.linspace(-1e-6, 1e-6, 2001)])
+    h = x.astype(np.float32).astype(np.float64)
+    x = h + (x - h).astype(np.float32)  # a pair
+    err = np.abs(_math(4, x).astype(L) - np.log(x.astype(L)))
+    print(f"\nln in double-float: {float(err.max()):.3g}")
+    assert err.max() <= 6 * 2.0**-46
