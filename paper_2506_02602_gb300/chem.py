@@ -28,6 +28,7 @@ NUM_ELEMENTS = 3
 OK, ERR_INVALID, ERR_CUDA, ERR_UNSUPPORTED, ERR_NOMEM, ERR_TIMEOUT, ERR_STATE = 0, -1, -2, -3, -4, -5, -6
 CELL_OK, CELL_MAX_STEPS, CELL_H_UNDERFLOW, CELL_NEWTON_FAIL, CELL_NONFINITE, CELL_SURROGATE = range(6)
 VARIANTS = {"fp64": 0, "mixed": 1}
+TRAIN_EPOCHS = 20  # of a chem_train_cfg with epochs 0
 SCHEMES = {"lsrk": 0, "full": 1, "rkf45": 2}
 
 
@@ -441,18 +442,18 @@ class Context:
     # learned surrogate ------------------------------------------------------------
     def surrogate_train(self, rho, e, Y0, dt, Y1, T0=None, epochs=20, batch=4096, lr=1e-3,
                         lr_final=0.0, boxcox_lambda=0.1, seed=0, dt_power=0.0, stream=None):
-        """chem_surrogate_train on CUDA tensors (Y0, Y1: [S, n] planes; dt: [n]).
-        Returns the mean loss of every epoch (numpy)."""
+        """chem_surrogate_train on CUDA tensors (Y0, Y1: [S, n] planes; dt: [n]); epochs 0 is the
+        library's default.  Returns the mean loss of every epoch (numpy)."""
         n = rho.numel()
         for nm, t in (("rho", rho), ("e", e), ("Y0", Y0), ("dt", dt), ("Y1", Y1)):
             _check_f64_cuda(nm, t, n)
         pr = Pairs(rho.data_ptr(), e.data_ptr(), Y0.data_ptr(), Y0.stride(0),
                    None if T0 is None else T0.data_ptr(), dt.data_ptr(), Y1.data_ptr(), Y1.stride(0))
         cfg = TrainCfg(epochs, batch, lr, lr_final, boxcox_lambda, dt_power, seed)
-        loss = np.zeros(max(epochs, 1), dtype=np.float32)
+        loss = np.zeros(epochs if epochs > 0 else TRAIN_EPOCHS, dtype=np.float32)
         self._raise(self.L.chem_surrogate_train(self.h, C.byref(pr), n, C.byref(cfg), _stream(stream),
                                                 loss.ctypes.data_as(C.c_void_p)))
-        return loss[:epochs]
+        return loss
 
     def surrogate_infer(self, rho, e, Y, T, dt, rtol=1e-6, atol=1e-10, status=None, nsteps=None,
                         mask=None, stats=None, gate=None, stream=None):
