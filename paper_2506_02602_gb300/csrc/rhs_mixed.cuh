@@ -165,8 +165,12 @@ __device__ __forceinline__ void load_mixed_tables(const MechTables &mt) {
   __syncthreads();
 }
 
-struct RateInputsF {
-  float lnT, invT, T, ctot;
+struct RateTempsF {
+  float lnT, invT, T;
+};
+// for the fp32 estimators
+struct RateInputsF : RateTempsF {
+  float ctot;
   float c[NSP];
 };
 
@@ -509,7 +513,7 @@ __device__ __forceinline__ float troe_rolled(float4 p, float n, float T, float i
 // Rate of progress (without the third-body factor) of fall-off reaction f (slot NRL + f) and of
 // the loop's reaction i; returns whether the exponent may round either way.
 template <int ST>
-__device__ __forceinline__ bool falloff_rate(int f, const RateInputsF &in, const float (&M)[NM], float2 rt,
+__device__ __forceinline__ bool falloff_rate(int f, const RateTempsF &in, const float (&M)[NM], float2 rt,
                                              const MixedCols &m) {
   const int i = NRL + f;
   const float4 k = s_rx_k[i], kk = s_rx_f[i], k0 = s_fo_k[f];
@@ -530,7 +534,7 @@ __device__ __forceinline__ bool loop_rate(int i, float lnT, float invT, float2 r
 
 // Every reaction's, rolled.  Returns the bits whose exponents may round either way.
 template <int ST>
-__device__ __forceinline__ unsigned all_rates(const RateInputsF &in, const float (&M)[NM], float2 rt, const MixedCols &m) {
+__device__ __forceinline__ unsigned all_rates(const RateTempsF &in, const float (&M)[NM], float2 rt, const MixedCols &m) {
   unsigned doubt = 0;
 #pragma unroll 1
   for (int f = 0; f < NFO; ++f)
@@ -542,7 +546,7 @@ __device__ __forceinline__ unsigned all_rates(const RateInputsF &in, const float
 }
 // Those of the bits in todo, out of line.
 template <int ST>
-static __device__ __noinline__ void some_rates(const RateInputsF *in, const float *M, float2 rt, unsigned todo) {
+static __device__ __noinline__ void some_rates(const RateTempsF *in, const float *M, float2 rt, unsigned todo) {
   const MixedCols m = mixed_cols<ST>();
   float Mr[NM];
 #pragma unroll
@@ -583,7 +587,7 @@ __device__ __forceinline__ void all_progress(const float *Q, const float (&M)[NM
 template <int ST>
 __device__ __forceinline__ bool cell_rhs_mixed(const MechTables &mt, const MixedCols &m, float rho_f, float invRho_f,
                                                ff eR, ff &T) {
-  RateInputsF in;
+  RateTempsF in;
   const ff guess = T;
   float2 rt = make_float2(0.0f, 0.0f);  // ln(R_u T / p_ref)
   constexpr unsigned kAll = (1u << NRX) - 1u;
@@ -625,7 +629,7 @@ __device__ __forceinline__ bool cell_rhs_mixed(const MechTables &mt, const Mixed
     Fp64Out o;
     if (!solve_gibbs_fp64<ST>(mt, m.CU, ff2d(eR), ff2d(guess), m.G, &o)) return false;
     T = ff_norm(d2ff(o.T));
-    RateInputsF in2;
+    RateTempsF in2;
     in2.T = d2f(o.T);
     in2.lnT = o.lnT;
     in2.invT = o.invT;
