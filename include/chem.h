@@ -72,9 +72,10 @@ typedef enum {
                              and end at 4e-10 T, within 1e-15 of the root) */
   CHEM_VARIANT_MIXED = 1  /* rates and RK stage derivatives in fp32; solution and error
                              registers and step control in fp64; temperature solve and Gibbs
-                             functions in double-float, redone in fp64 where the fp32 rounding
-                             of T, ln T, 1/T or ln(1/K_c) is in doubt; ln(1/K_c) is rounded
-                             once to fp32 for the fp32 reverse rate */
+                             functions in double-float (48 bits), or fp64 where their fp32
+                             rounding is close: T, ln T, 1/T and ln(1/K_c), each rounded once
+                             to fp32, are no further from the exact values than fp64 ones
+                             rounded once, but not always the same fp32 numbers */
 } chem_variant;
 
 /*
@@ -127,10 +128,10 @@ typedef struct {
   int32_t variant;     /* chem_variant [CHEM_VARIANT_FP64] */
   int32_t max_steps;   /* attempted-step limit per cell and call [100000] */
   int32_t block_size;  /* threads per block of the one-pass integration kernel: 32, 64
-                          (16 warps per SM, 128 registers a thread; 64 registers for the
-                          mixed two-register scheme), 128 (12 warps, 170 registers; mixed
-                          two-register scheme with 9 species: 16 warps, 128 registers) or
-                          256 (8 warps, 255 registers); other values take 128 [0: 128] */
+                          (at most 128 registers a thread; 64 for the mixed two-register
+                          scheme), 128 (170; mixed two-register scheme with 9 species: 128)
+                          or 256 (255); other values take 128 [0: 128].  Shared memory leaves
+                          about 5 to 12, 8 to 14, 8 to 16 and 8 warps per SM */
   int32_t scheme;      /* chem_scheme [CHEM_SCHEME_LSRK]; the comparators serve
                           chem_integrate and chem_integrate_host only: the batched and
                           surrogate calls of a context with another scheme return
@@ -252,8 +253,9 @@ typedef struct {
   const int32_t *d_box_nsub;
 } chem_batch;
 
-/* Compiled shapes of the persistent kernel: (threads per CTA, minimum resident CTAs
- * per SM, hence a register cap of min(255, 65536 / (threads * CTAs))):
+/* Compiled shapes of the persistent kernel: (threads per CTA, CTAs per SM that its
+ * registers are capped for, min(255, 65536 / (threads * CTAs)) each; shared memory may hold
+ * fewer, chem_batch_shape_info tells):
  * 0 = (128, 3) [default], 1 = (128, 2), 2 = (128, 4), 3 = (64, 6), 4 = (64, 8), 5 = (256, 2)
  * for fp64; for the mixed variant 0 = (128, 4) [default; (128, 3) with 13 species],
  * 1 = (128, 3), 2 = (128, 2) and 4 = (64, 16) ((64, 8) with 13 species), the others as for fp64.

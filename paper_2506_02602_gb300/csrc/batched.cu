@@ -8,7 +8,7 @@
 //
 //   1. k_probe: a stiffness key per cell -- the caller's cost hint (for example the
 //      attempted steps of the previous call), or one fp32 right-hand side (in fp64 it took
-//      14 of the 3.5 M-cell AMR batch's 70 ms) giving an accuracy estimate (dt max|F| / tol)^(1/4) and a stability estimate
+//      10 of the 3.5 M-cell AMR batch's 70 ms) giving an accuracy estimate (dt max|F| / tol)^(1/4) and a stability estimate
 //      dt max_k (consumption rate of k / c_k) / 3 -- times the box's substeps, binned
 //      into half-octave buckets with a block histogram;
 //   2. k_scan + k_scatter: a counting sort of the cell indices into descending-cost
@@ -202,10 +202,12 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_lsrk_persistent(const __grid_co
   if (a.stats) accumulate_stats(a.stats, done_cells, tot_acc, tot_rej, tot_rhs, max_steps, hist);
 }
 
-// Threads per CTA and minimum resident CTAs per SM of each shape; shape 0 is the default.  fp64: 12
-// warps per SM run the 3.46 M-cell ragged AMR batch in 255 ms, 8 (128 x 2, which had no spills
-// when a cell's vectors were in registers) in 280, and the 128-register shapes in 259 to 297.
-// Mixed: its per-thread columns allow 16 warps (12 with 13 species), 59 ms against 65 at 12 and 80
+// Threads per CTA and CTAs per SM that the registers are capped for, of each shape; shape 0 is the
+// default.  Shared memory (per-thread columns and tables) holds fewer CTAs than that in fp64 of shapes
+// 2 to 4 (3, 5, 5) and with 13 species (2, 2, 2, 4, 4, 1), and of the mixed shape 4 (7 of 16).  fp64: 12
+// warps per SM run the 3.46 M-cell ragged AMR batch in 179 ms, 8 (128 x 2) in 196, and the
+// 128-register shapes in 178 to 204.
+// Mixed: the columns allow 16 warps (12 with 13 species), 59 ms against 65 at 12 and 80
 // at 8 (and 73 for the 64-register shape 4).
 static constexpr int kShapeBlock[CHEM_BATCH_SHAPES] = {128, 128, 128, 64, 64, 256};
 template <int V>
@@ -307,7 +309,7 @@ cudaError_t launch_persistent_queue(int variant, const MechTables &mt, const Bat
   if (a.n <= 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
-  const int shape = 0;  // the fastest of each variant on the ragged AMR batch
+  const int shape = 0;  // within 1 % of the fastest of each variant on the ragged AMR batch
   int sms = 0, pblock = 0, per = 0, regs = 0;
   e = persistent_shape(variant, shape, &pblock, &per, &regs, &sms);
   if (e != cudaSuccess) return e;

@@ -7,7 +7,8 @@
 
 namespace chem {
 
-// BLOCK threads per block, MINB resident blocks per SM.  The register file is split
+// BLOCK threads per block; the registers are capped for MINB resident blocks per SM, which shared memory
+// (per-thread columns and tables) may not hold.  The register file is split
 // between the SM's four sub-partitions, so 12 warps per SM allow 170 registers a thread
 // (128 x 3), 16 warps 128 (64 x 8, 32 x 16, 128 x 4) and 32 warps 64 (64 x 16, 32 x 32);
 // anything between rounds down; 8 warps (256 x 1) leave the 255-register maximum.
@@ -84,12 +85,14 @@ static cudaError_t launch_one(const MechTables &mt, const CellArgs &a, const Ste
   return cudaGetLastError();
 }
 
-// The compiled shapes.  fp64: 12 warps per SM (128 x 3, 168 registers, no spills) runs the
-// 1M-cell detonation slice in 26.1 ms, 64 threads (128 registers; the columns and the 23 KB of
-// tables leave 10 warps) in 28.6, 32 threads in 37.1 and 8 warps (256) in 31.7.  The mixed two-register kernel's per-thread columns allow 16 warps
-// per SM (12 with 13 species): 128 x 4 at 128 registers, 7.9 ms on the 1M-cell detonation slice;
-// its 32- and 64-thread shapes keep 64 registers (14 warps of 64 threads, spilling): 9.3 ms at
-// 64, 11.2 at 32.
+// The compiled shapes.  fp64: 12 warps per SM (128 x 3, 146 registers, no spills) run the
+// 1M-cell detonation slice in 24.9 ms, 64 threads (128 registers; the columns and the 23 KB of
+// tables leave 10 warps) in 26.2, 32 threads in 33.7 and 8 warps (256) in 30.6.  With 13 species the
+// columns leave 8 warps at 128 and at 64 threads: 6.9 and 6.4 ms on 401 x 379 cells.  The mixed
+// two-register kernel's per-thread columns allow 16 warps
+// per SM (12 with 13 species): 128 x 4 at 128 registers, 8.0 ms on the 1M-cell detonation slice;
+// its 32- and 64-thread shapes keep 64 registers (14 warps of 64 threads, spilling): 9.4 ms at
+// 64, 11.2 at 32, and 13.2 at 256 (8 warps).
 template <int V, int SCH>
 static cudaError_t launch_shape(const MechTables &mt, const CellArgs &a, const StepParams &p, int block,
                                 cudaStream_t s) {

@@ -40,7 +40,7 @@ namespace {
 constexpr int GM = 128;      // rows per CTA tile (MMA M)
 constexpr int GKC = 64;      // K of a staged chunk
 constexpr int GNMAX = 64;    // widest N tile (MMA N): 256-wide outputs run as 4 tiles, 4x the CTAs
-constexpr int GTHR = 512;    // 16 warps: 4 per accumulator lane quarter, each a quarter of the columns
+constexpr int GTHR = 512;    // 16 warps: 4 per accumulator lane quarter, each half of the columns and of the rows
 constexpr uint32_t kStageA = GM * GKC * 2;            // 16 KB
 constexpr uint32_t kStageB = GNMAX * GKC * 2;         // 8 KB
 constexpr uint32_t kStage = kStageA + kStageB;

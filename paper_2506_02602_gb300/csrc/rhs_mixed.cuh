@@ -10,11 +10,15 @@
 //         rates and F.
 // What reaches the fp32 part is T, ln T, 1/T and the equilibrium exponents
 // ln(1 / K_c,j) = sum_k nu_jk g_k + (sum_k nu_jk) ln(R_u T / p_ref), each rounded once to
-// fp32.  Those are meant to be the fp64 values rounded once, and a rounding test (Ziv,
-// ACM TOMS 17 (1991) 410-423) makes them so: where the double-float value lies within its
-// error of the middle between two fp32 numbers, the cell's temperature and Gibbs functions
+// fp32.  They are to be no less exact than fp64 values rounded once, and a rounding test (Ziv,
+// ACM TOMS 17 (1991) 410-423) sees to it: where the double-float value lies near the middle between
+// two fp32 numbers, the cell's temperature and Gibbs functions
 // are evaluated again in fp64 (solve_gibbs_fp64; 0.4 % of the cells' evaluations).
-// The exponents are summed from fp32 hi parts on a 2^-12 grid (exact in fp32) and lo parts.
+// The exponents are summed from fp32 hi parts on a 2^-12 grid (exact in fp32) and lo parts, in fp64
+// as here; it is the lo parts' rounding that limits both.  Over 200,000 temperatures from 250 to
+// 4500 K an exponent of fp64 Gibbs functions is up to 4.6e-11 beyond half an fp32 ulp off, one of
+// double-float functions 5.4e-11, and one that passed the test, at kLnKcErr = 2.4e-11, thus at most
+// 3.0e-11.  (The two are still other fp32 numbers now and then, neither of them nearer: see there.)
 //
 // On GB300 an FP64 instruction costs a warp 64 cycles of its sub-partition whatever else the
 // warp does, a double-float multiply-add about 13 (6 with the packed f32x2 forms).  With the
@@ -22,7 +26,7 @@
 // slots 26 %; now the pipe is 51 % busy (the solution and error registers, the norm, the
 // evaluations in fp64) and issue 53 %.  What bounds the kernel is the latency of dependent
 // fp32 operations at 16 warps an SM, and it runs the 1M-cell detonation slice in 7.9 ms
-// instead of 16.1 (the 151,979-cell 13-species slice in 2.1 instead of 3.4).
+// instead of 16.1 (the 151,979-cell 13-species slice in 2.46 instead of 3.40).
 //
 // Straight-line code is fetched at no more than two instructions a clock and SM, and code that
 // exceeds the instruction caches (the unrolled form: 64 KB) at the speed of the L2; so the
@@ -459,9 +463,10 @@ __device__ __forceinline__ bool solve_T_ff(const MechTables &mt, const float2 *C
 
 // Rounding test of the exponents: the double-float sums are within ~2e-12 of the fp64
 // ones, but their lo parts may round to the other neighbour on the 2^-36 grid that fp32 gives
-// them (four terms, seldom more than one of them); kLnKcErr covers that.  On an AMR batch of
-// 3.5 M cells (65 evaluations a cell and more) 1.6e-11 leaves 110 cells with another rounding
-// somewhere, 2.4e-11 40 and 4e-11 15; each step costs about 4 % of the kernel's time.
+// them (four terms, seldom more than one of them); kLnKcErr covers one of them, not several at
+// once.  On an AMR batch of 3.5 M cells (65 evaluations a cell and more) 1.6e-11 leaves 110 cells
+// in which some exponent is another fp32 number than from fp64 functions, 2.4e-11 40 and 4e-11 15;
+// each step costs about 4 % of the kernel's time.
 constexpr float kLnKcErr = 2.4e-11f;
 
 // k_f c_r0 c_r1 - k_r c_p0 c_p1 with k_r = exp(ln k_f + ln(1 / K_c)), k_f > t else 0, given
