@@ -36,7 +36,9 @@ GPU integrator, 2M (state, dt ~ logU[1e-9, 1e-7] s) -> state training pairs from
 them, training on the GPU (batch 4096), and inference on 16,777,216 cells drawn from the
 held-out 10 %, against plain fp64 and mixed integration of the same cells.
 
-Legs of one run (rank 0 prints one JSON line):
+Rank 0 prints one JSON line of a few KB with the headline and one figure of each leg; the whole
+result (every variant, leg and candidate, some 35 KB) goes to the file of --detail, which the line
+names.  Legs of one run:
   surrogate data generation, training and inference (above; skipped by --no-surrogate,
             which also drops the hybrid variant);
   value     device-resident throughput (cells/s) of the headline variant;
@@ -76,8 +78,52 @@ def _jsonable(o):
     raise TypeError(f"not serialisable: {type(o).__name__}")
 
 
+HEADLINE_KEYS = ("impl", "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better",
+                 "scaling", "vs_baseline", "dtype", "data", "config", "kernel_ms", "roofline", "e2e", "gpu_launches",
+                 "clocks", "cpu_baseline")
+# one figure of each leg: its name in the line, and where it is in the whole result
+LEG_FIGURES = {
+    "reactors_4096_fp64_ms": ("reactors_4096", "ms"),
+    "amr_256_boxes_fp64_ms": ("amr_batch", "fp64", "persistent_ms"),
+    "amr_256_boxes_mixed_ms": ("amr_batch", "mixed", "persistent_ms"),
+    "mech13_fp64_ms": ("mech13", "fp64", "ms"),
+    "mech13_mixed_ms": ("mech13", "mixed", "ms"),
+}
+VARIANT_KEYS = ("value", "kernel_ms", "meets_stated_error", "stated_error_T", "error_vs_fp64_gpu", "roofline_frac")
+
+
+def headline(result, detail=None):
+    """The printed line: the contract's keys, each variant's and each leg's main figures, and the
+    file of the whole result.  A line of the whole result was cut to its end wherever output is
+    kept by its tail."""
+    line = {k: result[k] for k in HEADLINE_KEYS if k in result}
+    line["variants"] = {v: {k: d[k] for k in VARIANT_KEYS if k in d} for v, d in (result.get("variants") or {}).items()}
+    figures = {}
+    for name, path in LEG_FIGURES.items():
+        at = result
+        for k in path:
+            at = at.get(k) if isinstance(at, dict) else None
+        if at is not None:
+            figures[name] = at
+    line["legs"] = figures
+    line["detail"] = detail
+    return line
+
+
+def write_detail(result, path):
+    """The whole result into the file; its path, or None where it cannot be written."""
+    try:
+        with open(path, "w") as f:
+            json.dump(result, f, default=_jsonable)
+            f.write("\n")
+    except OSError:
+        return None
+    return path
+
+
 def parse():
     ap = argparse.ArgumentParser()
+    ap.add_argument("--detail", default=os.path.join(ROOT, "bench_detail.json"), help="file of the whole result")
     ap.add_argument("--gpus", type=int, default=1)
     ap.add_argument("--steps", type=int, default=20)
     ap.add_argument("--warmup", type=int, default=3)
@@ -1198,7 +1244,7 @@ def run_ours(args, rank, world, local):
             "cpu_baseline_configs": cpu_cfgs,
             "parity_vs_oracle_sample": parity,
         }
-        print(json.dumps(line, default=_jsonable), flush=True)
+        print(json.dumps(headline(line, write_detail(line, args.detail)), default=_jsonable), flush=True)
     for c in ctxs.values():
         c.close()
     if world > 1:
