@@ -381,8 +381,8 @@ MLP_FLOPS_PER_ROW = 2 * (16 * 256 + 256 * 256 * 2 + 256 * 16)  # padded 16-256-2
 # DRAM bytes (read + write) per cell of one k_lsrk launch (dram__bytes_read.sum +
 # dram__bytes_write.sum), from an ncu capture of the 131,072-cell slice, scaled by the
 # cell count; to be set to None whenever the kernel changes until it is captured again.
-# fp64: 12.95 MB read per 131,072-cell launch, mixed: 13.87 MB read + 0.26 MB written
-TRAFFIC_PER_CELL = {"fp64": 12.95e6 / 131072, "mixed": 14.13e6 / 131072}
+# fp64: 12.95 MB read per 131,072-cell launch, mixed: 13.75 MB read + 0.23 MB written
+TRAFFIC_PER_CELL = {"fp64": 12.95e6 / 131072, "mixed": 13.98e6 / 131072}
 
 
 def _bf16_peak():
