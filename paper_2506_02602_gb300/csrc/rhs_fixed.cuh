@@ -18,7 +18,7 @@
 // A warp's evaluation issued 1040 FP64 instructions in the general form, 637 with only its
 // exponentials in fixed point and 300 here; the 1M-cell detonation slice takes 83.2, 49.2 and
 // 24.9 ms, a 256-cell batch of 15 steps 3.0, 2.1 and 1.3 ms (one warp's chain of dependent
-// instructions).  Integer work now fills the issue slots the FP64 pipe (70 % busy) leaves.
+// instructions).  Integer work now fills the issue slots the FP64 pipe (72 % busy) leaves.
 //
 // For T in (128, 8192) K, |Y_k| < 1.25, sum |Y_k| <= 1.5, |e| / R_u < 2^26 K mol/kg, rho in
 // (2^-64, 2^64) and coefficients within the tables' ranges (MechTables::fixed_ok); anything else takes
